@@ -946,6 +946,48 @@ void launch_bicg_xr(const Grid& G, const V2<T>* ph, const V2<T>* sh,
     k_bicg_xr<T><<<grid, kBS, 0, st>>>(G.N, ph, sh, s, t, rh, x, r, partial, ks);
 }
 
+// Threads of a block that sums nblk partials of one sample: about 8 partials
+// per thread (two batches of 4 loads in flight), at most 1024 threads.  A
+// block's time is its number of dependent load batches: at 256x256x64 the
+// products leave 134 k partials per sum, which 128 threads read in 1,048
+// dependent rounds (391 us); 1024 threads with 4 loads in flight need 33.
+// Two samples of that grid: 302 -> 233 ms per step; one at 128x128x32: 30.3 ->
+// 27.3 ms.
+inline int finalize_threads(int nblk)
+{
+    int t = 128;
+    while (t < 1024 && 8 * t < nblk) t *= 2;
+    return t;
+}
+
+// This thread's share of sum_q v[q], q < n, in four independent partial sums.
+__device__ __forceinline__ double strided_sum(const double* __restrict__ v, int n)
+{
+    double a[4] = {0.0, 0.0, 0.0, 0.0};
+    const int st = blockDim.x;
+    int q = threadIdx.x;
+    for (; q + 3 * st < n; q += 4 * st) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) a[u] += v[q + u * st];
+    }
+    for (; q < n; q += st) a[0] += v[q];
+    return (a[0] + a[1]) + (a[2] + a[3]);
+}
+
+// This thread's share of the larger of 0 and max_q v[q], q < n.
+__device__ __forceinline__ double strided_max(const double* __restrict__ v, int n)
+{
+    double a[4] = {0.0, 0.0, 0.0, 0.0};
+    const int st = blockDim.x;
+    int q = threadIdx.x;
+    for (; q + 3 * st < n; q += 4 * st) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) a[u] = fmax(a[u], v[q + u * st]);
+    }
+    for (; q < n; q += st) a[0] = fmax(a[0], v[q]);
+    return fmax(fmax(a[0], a[1]), fmax(a[2], a[3]));
+}
+
 // One block per sample: fixed-order sums of the partials and the BiCGStab
 // scalar recurrences.
 __global__ void k_bicg_finalize(int stage, const double* __restrict__ partial,
@@ -955,13 +997,12 @@ __global__ void k_bicg_finalize(int stage, const double* __restrict__ partial,
     const int s = blockIdx.x;
     KScal k = ks[s];
     if (!k.active) return;
-    double a0 = 0.0, a1 = 0.0;
-    for (int q = threadIdx.x; q < nblk; q += blockDim.x) {
-        a0 += partial[((size_t)s * 2 + 0) * nblk + q];
-        a1 += partial[((size_t)s * 2 + 1) * nblk + q];
-    }
+    // (stages 0 and 1 have one inner product; the second array is not written)
+    const bool two = stage >= 2;
+    double a0 = strided_sum(partial + ((size_t)s * 2 + 0) * nblk, nblk);
+    double a1 = two ? strided_sum(partial + ((size_t)s * 2 + 1) * nblk, nblk) : 0.0;
     a0 = block_sum(a0, red);
-    a1 = block_sum(a1, red);
+    if (two) a1 = block_sum(a1, red);
     if (threadIdx.x != 0) return;
     if (stage == 0) {  // after init: ||b||^2 = (rh, r)
         k.bn2 = a0;
@@ -1024,7 +1065,7 @@ void launch_bicg_finalize(int stage, const double* partial, int nblk,
                           cudaStream_t st)
 {
     count_launch(1);
-    k_bicg_finalize<<<S, 128, 0, st>>>(stage, partial, nblk, ks, rtol, maxit);
+    k_bicg_finalize<<<S, finalize_threads(nblk), 0, st>>>(stage, partial, nblk, ks, rtol, maxit);
 }
 
 template <class T>
@@ -1067,11 +1108,8 @@ __global__ void k_norm_finalize(const double* __restrict__ partial,
     const int s = blockIdx.x;
     if (which == 1 && !ns[s].ls_active) return;
     if (which == 0 && !ns[s].active) return;
-    double a = 0.0, b = 0.0;
-    for (int q = threadIdx.x; q < nblk; q += blockDim.x) {
-        a += partial[(size_t)s * nblk + q];
-        if (act) b += act[(size_t)s * nblk + q];
-    }
+    double a = strided_sum(partial + (size_t)s * nblk, nblk);
+    double b = act ? strided_sum(act + (size_t)s * nblk, nblk) : 0.0;
     a = block_sum(a, red);
     b = block_sum(b, red);
     if (threadIdx.x != 0) return;
@@ -1099,7 +1137,7 @@ void launch_norm_finalize(const double* partial, const double* act, int nblk, NS
                           int which, int S, cudaStream_t st)
 {
     count_launch(1);
-    k_norm_finalize<<<S, 128, 0, st>>>(partial, act, nblk, ns, which);
+    k_norm_finalize<<<S, finalize_threads(nblk), 0, st>>>(partial, act, nblk, ns, which);
 }
 
 template <class T>
@@ -1205,11 +1243,8 @@ __global__ void k_newton_ls_finalize(const double* __restrict__ pmax, int nblk,
     __shared__ double red[32];
     const int s = blockIdx.x;
     if (!ns[s].ls_active) return;
-    double a0 = 0.0, a1 = 0.0;
-    for (int q = threadIdx.x; q < nblk; q += blockDim.x) {
-        a0 = fmax(a0, pmax[((size_t)s * 2 + 0) * nblk + q]);
-        a1 = fmax(a1, pmax[((size_t)s * 2 + 1) * nblk + q]);
-    }
+    double a0 = strided_max(pmax + ((size_t)s * 2 + 0) * nblk, nblk);
+    double a1 = strided_max(pmax + ((size_t)s * 2 + 1) * nblk, nblk);
     a0 = block_max(a0, red);
     a1 = block_max(a1, red);
     if (threadIdx.x != 0) return;
@@ -1240,7 +1275,7 @@ void launch_newton_ls_finalize(const double* partial_res,
 {
     count_launch(1);
     (void)partial_res;
-    k_newton_ls_finalize<<<S, 128, 0, st>>>(partial_max, nblk, ns, ls_max);
+    k_newton_ls_finalize<<<S, finalize_threads(nblk), 0, st>>>(partial_max, nblk, ns, ls_max);
 }
 
 __global__ void __launch_bounds__(kBS)
@@ -1299,11 +1334,8 @@ __global__ void k_newton_predict(const double* __restrict__ pmax, int nblk, NSca
     __shared__ double red[32];
     const int s = blockIdx.x;
     if (!ns[s].ls_active || ns[s].lambda != 1.0) return;
-    double a0 = 0.0, a1 = 0.0;
-    for (int q = threadIdx.x; q < nblk; q += blockDim.x) {
-        a0 = fmax(a0, pmax[((size_t)s * 2 + 0) * nblk + q]);
-        a1 = fmax(a1, pmax[((size_t)s * 2 + 1) * nblk + q]);
-    }
+    double a0 = strided_max(pmax + ((size_t)s * 2 + 0) * nblk, nblk);
+    double a1 = strided_max(pmax + ((size_t)s * 2 + 1) * nblk, nblk);
     a0 = block_max(a0, red);
     a1 = block_max(a1, red);
     if (threadIdx.x != 0) return;
@@ -1322,7 +1354,7 @@ void launch_newton_predict(const double* partial_max, int nblk, NScal* ns, doubl
                            double tol_c, int estimate, int S, cudaStream_t st)
 {
     count_launch(1);
-    k_newton_predict<<<S, 128, 0, st>>>(partial_max, nblk, ns, tol_p, tol_c, estimate);
+    k_newton_predict<<<S, finalize_threads(nblk), 0, st>>>(partial_max, nblk, ns, tol_p, tol_c, estimate);
 }
 
 __global__ void k_newton_check(NScal* ns, const KScal* ks, double tol_p,
@@ -1481,8 +1513,7 @@ __global__ void k_sum_partials(const double* __restrict__ partial, int nblk,
                                double* __restrict__ out)
 {
     __shared__ double red[32];
-    double a = 0.0;
-    for (int q = threadIdx.x; q < nblk; q += blockDim.x) a += partial[(size_t)blockIdx.x * nblk + q];
+    double a = strided_sum(partial + (size_t)blockIdx.x * nblk, nblk);
     a = block_sum(a, red);
     if (threadIdx.x == 0) out[blockIdx.x] = a;
 }
@@ -1491,7 +1522,7 @@ void launch_sum_partials(const double* partial, int nblk, double* out, int S,
                          cudaStream_t st)
 {
     count_launch(1);
-    k_sum_partials<<<S, 128, 0, st>>>(partial, nblk, out);
+    k_sum_partials<<<S, finalize_threads(nblk), 0, st>>>(partial, nblk, out);
 }
 
 // which = 0: y = a x on Dirichlet components only, 0 elsewhere;
