@@ -16,6 +16,11 @@
 //
 // Every node kernel gathers the contributions of the up to 8 cells around
 // its node (one thread per node, no atomics, deterministic).
+#include <cooperative_groups.h>
+
+#include <type_traits>
+#include <utility>
+
 #include "kernels.h"
 
 namespace elder {
@@ -831,149 +836,312 @@ void launch_average_cells(const Grid& Gf, const Grid& Gc, const double* phif,
 }
 
 // ---------------------------------------------------------------------------
-// coarsest level: dense inverse of the interior operator (Gauss-Jordan with
-// partial pivoting, FP64), one block per sample.  work: [S][n][2n].
+// coarsest level: dense inverse of the interior operator by in-place
+// Gauss-Jordan elimination with partial pivoting.  The rows are not exchanged:
+// step k takes the largest entry of column k among the rows not yet used as
+// pivots, row p_k; afterwards M[i][j] holds Ainv[k(i)][p_j], k(i) the step at
+// which row i was the pivot.  A column with no entry but its pivot (the
+// Dirichlet unknowns, about a third of the 4x4x1 grid's) only scales its row.
+// The inverse is stored by columns, Ainv[q][r] = (A^{-1})_{rq}: the plain
+// product reads it coalesced.
 // ---------------------------------------------------------------------------
 
+// Entries of the interior operator (Dirichlet rows and columns replaced by the
+// identity) in the columns [c0, c1), written to A[row * ld + col - c0]; A has
+// been zeroed.
 template <class M, class R>
-__global__ void k_coarse_build(Grid G, const uint8_t* __restrict__ bc,
-                               const B4<M>* __restrict__ J, R* __restrict__ W,
-                               const int* mask, int mstride)
+__device__ __forceinline__ void coarse_fill(const Grid& G, const uint8_t* __restrict__ bc,
+                                            const B4<M>* __restrict__ J, R* A, int ld, int c0,
+                                            int c1)
 {
-    const int s = blockIdx.y;
-    if (!sample_on(mask, mstride, s)) return;
-    const int node = blockIdx.x * blockDim.x + threadIdx.x;
-    if (node >= G.N) return;
-    const int n2 = 2 * G.N;
-    R* row0 = W + (size_t)s * n2 * 2 * n2 + (size_t)(2 * node) * 2 * n2;
-    R* row1 = row0 + 2 * n2;
-    for (int q = 0; q < 2 * n2; ++q) { row0[q] = R(0); row1[q] = R(0); }
-    int i, j, k;
-    node_ijk(G, node, i, j, k);
-    const uint8_t mr = bc[node];
-    for (int dz = -1; dz <= 1; ++dz)
-        for (int dy = -1; dy <= 1; ++dy)
-            for (int dx = -1; dx <= 1; ++dx) {
-                const int ii = i + dx, jj = j + dy, kk = k + dz;
-                if (ii < 0 || ii > G.nx || jj < 0 || jj > G.ny || kk < 0 || kk > G.nz)
-                    continue;
-                const int m = node_id(G, ii, jj, kk);
-                const uint8_t mc = bc[m];
-                const B4<M> B = J[((size_t)s * 27 + slot27(dx, dy, dz)) * G.N + node];
-                if (!(mr & BC_P)) {
-                    if (!(mc & BC_P)) row0[2 * m] = mg_load<R>(B.pp);
-                    if (!(mc & BC_C)) row0[2 * m + 1] = mg_load<R>(B.pc);
-                }
-                if (!(mr & BC_C)) {
-                    if (!(mc & BC_P)) row1[2 * m] = mg_load<R>(B.cp);
-                    if (!(mc & BC_C)) row1[2 * m + 1] = mg_load<R>(B.cc);
-                }
+    for (int e = threadIdx.x; e < 27 * G.N; e += blockDim.x) {
+        const int slot = e / G.N, node = e - slot * G.N;
+        const int dx = slot % 3 - 1, dy = (slot / 3) % 3 - 1, dz = slot / 9 - 1;
+        int i, j, k;
+        node_ijk(G, node, i, j, k);
+        if (i + dx < 0 || i + dx > G.nx || j + dy < 0 || j + dy > G.ny || k + dz < 0 ||
+            k + dz > G.nz)
+            continue;
+        const int m = node_id(G, i + dx, j + dy, k + dz);
+        const uint8_t mr = bc[node], mc = bc[m];
+        const B4<M> B = J[(size_t)slot * G.N + node];
+        R v[2][2] = {{mg_load<R>(B.pp), mg_load<R>(B.pc)}, {mg_load<R>(B.cp), mg_load<R>(B.cc)}};
+#pragma unroll
+        for (int a = 0; a < 2; ++a)
+#pragma unroll
+            for (int b = 0; b < 2; ++b) {
+                const int c = 2 * m + b;
+                if (c < c0 || c >= c1) continue;
+                const bool dr = (mr >> a) & 1, dc = (mc >> b) & 1;
+                R x = v[a][b];
+                if (dr || dc) x = (slot == 13 && a == b) ? R(1) : R(0);
+                A[(size_t)(2 * node + a) * ld + c - c0] = x;
             }
-    if (mr & BC_P) row0[2 * node] = R(1);
-    if (mr & BC_C) row1[2 * node + 1] = R(1);
-    row0[n2 + 2 * node] = R(1);
-    row1[n2 + 2 * node + 1] = R(1);
+    }
 }
 
-// Gauss-Jordan with partial pivoting on [A | I] of one sample per block, in
-// arithmetic R (FP32 for the mixed solver, whose coarse matrix is stored in
-// bfloat16 and is only a preconditioner; FP64 otherwise).  SMEM: the
-// augmented matrix is copied into shared memory first (it fits for the
-// 100-unknown 4x4x1 coarsest grid), which keeps the n elimination sweeps
-// off L2; otherwise it is eliminated in place in global memory.  Each warp
-// updates whole rows, columns k..2n-1 only.
-template <bool SMEM, class R>
-__global__ void k_gauss_jordan(int n, R* __restrict__ W, R* __restrict__ Ainv, const int* mask,
-                               int mstride)
+// Pivot of a step: the largest |col[i]| over the rows not yet used (the lowest
+// of equal ones) and whether another row has an entry.  Called by one warp;
+// used: bit q of lane l is row l + 32 q.
+template <class R>
+__device__ __forceinline__ int gj_pivot(const R* col, int n, unsigned long long used, bool& other)
+{
+    const int lane = threadIdx.x & 31;
+    R best = R(-1);
+    int bi = 0x7fffffff;  // (a lane without an unused row)
+    int cnt = 0;
+    for (int q = 0, i = lane; i < n; ++q, i += 32) {
+        R a = fabs(col[i]);
+        cnt += a != R(0) ? 1 : 0;
+        if (a != a) a = R(INFINITY);  // a NaN is a pivot like any other: all lanes agree
+        if (!((used >> q) & 1) && a > best) { best = a; bi = i; }
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        const R ob = __shfl_xor_sync(0xffffffffu, best, o);
+        const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+        if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
+    }
+    other = __reduce_add_sync(0xffffffffu, (unsigned)cnt) > 1u;
+    return bi;
+}
+
+// The 16 steps of register slot b0 (a compile-time index, so that v stays in
+// registers).
+template <int NB, int b0>
+__device__ __forceinline__ void gj_panel(float (&v)[NB][NB], int n, float* col, float* row,
+                                         int* piv, int* inv_piv, volatile int* sp,
+                                         volatile int* sother, unsigned long long& used)
+{
+    const int tid = threadIdx.x, ti = tid >> 4, tj = tid & 15, lane = tid & 31;
+    for (int kk = 0; kk < 16 && 16 * b0 + kk < n; ++kk) {
+        const int k = 16 * b0 + kk;
+        if (tj == kk) {
+#pragma unroll
+            for (int a = 0; a < NB; ++a) col[ti + 16 * a] = v[a][b0];
+        }
+        __syncthreads();
+        if (tid < 32) {
+            bool other;
+            const int p = gj_pivot(col, n, used, other);
+            if (lane == (p & 31)) used |= 1ull << (p >> 5);
+            if (lane == 0) {
+                *sp = p;
+                *sother = other;
+                piv[k] = p;
+                inv_piv[p] = k;
+            }
+        }
+        __syncthreads();
+        const int p = *sp;
+        const bool other = *sother != 0;
+        const float inv = 1.f / col[p];
+        if (tj == kk) {
+#pragma unroll
+            for (int a = 0; a < NB; ++a) v[a][b0] = (ti + 16 * a == p) ? 1.f : 0.f;
+        }
+        if (ti == (p & 15)) {
+            // (selects: an indexed register would move v to local memory)
+            const int pa = p >> 4;
+#pragma unroll
+            for (int b = 0; b < NB; ++b) {
+                float x = v[0][b];
+#pragma unroll
+                for (int a = 1; a < NB; ++a) x = a == pa ? v[a][b] : x;
+                x *= inv;
+#pragma unroll
+                for (int a = 0; a < NB; ++a) v[a][b] = a == pa ? x : v[a][b];
+                row[tj + 16 * b] = x;
+            }
+        }
+        if (other) {  // (the same for every thread)
+            __syncthreads();
+            float r[NB];
+#pragma unroll
+            for (int b = 0; b < NB; ++b) r[b] = row[tj + 16 * b];
+#pragma unroll
+            for (int a = 0; a < NB; ++a) {
+                const int i = ti + 16 * a;
+                const float f = i == p ? 0.f : col[i];
+#pragma unroll
+                for (int b = 0; b < NB; ++b) v[a][b] = fmaf(-f, r[b], v[a][b]);
+            }
+        }
+        __syncthreads();  // col, row and the pivot are read
+    }
+}
+
+template <int NB, int... B>
+__device__ __forceinline__ void gj_panels(float (&v)[NB][NB], int n, float* col, float* row,
+                                          int* piv, int* inv_piv, volatile int* sp,
+                                          volatile int* sother, unsigned long long& used,
+                                          std::integer_sequence<int, B...>)
+{
+    (gj_panel<NB, B>(v, n, col, row, piv, inv_piv, sp, sother, used), ...);
+}
+
+// FP32, n <= 16 NB: one CTA per sample, the matrix in registers, thread
+// (ti, tj) of 16 x 16 holding the entries (ti + 16 a, tj + 16 b).  A step
+// shares the pivot column and the scaled pivot row through shared memory: two
+// barriers.
+template <class M, int NB>
+__global__ void __launch_bounds__(256)
+    k_gauss_jordan_reg(Grid G, const uint8_t* __restrict__ bc, const B4<M>* __restrict__ J,
+                       float* __restrict__ Ainv, const int* mask, int mstride)
 {
     extern __shared__ __align__(16) unsigned char gj_smem[];
-    __shared__ R rv[32];
-    __shared__ int ri[32];
     const int s = blockIdx.x;
     if (!sample_on(mask, mstride, s)) return;
-    const int w2 = 2 * n;
-    R* f = reinterpret_cast<R*>(gj_smem);
-    R* A = W + (size_t)s * n * w2;
-    if (SMEM) {
-        R* As = f + n;
-        for (int q = threadIdx.x; q < n * w2; q += blockDim.x) As[q] = A[q];
-        A = As;
-        __syncthreads();
-    }
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int n = 2 * G.N;
+    float* st = reinterpret_cast<float*>(gj_smem);  // [n][n], for the set-up
+    __shared__ float col[16 * NB], row[16 * NB];
+    __shared__ int piv[16 * NB], inv_piv[16 * NB];
+    __shared__ int sp, sother;
+    const int tid = threadIdx.x, ti = tid >> 4, tj = tid & 15;
+    for (int e = tid; e < n * n; e += blockDim.x) st[e] = 0.f;
+    __syncthreads();
+    coarse_fill<M, float>(G, bc, J + (size_t)s * 27 * G.N, st, n, 0, n);
+    __syncthreads();
+    float v[NB][NB];
+#pragma unroll
+    for (int a = 0; a < NB; ++a)
+#pragma unroll
+        for (int b = 0; b < NB; ++b) {
+            const int i = ti + 16 * a, j = tj + 16 * b;
+            v[a][b] = (i < n && j < n) ? st[i * n + j] : 0.f;
+        }
+    unsigned long long used = 0;  // (warp 0)
+    gj_panels<NB>(v, n, col, row, piv, inv_piv, &sp, &sother, used,
+                  std::make_integer_sequence<int, NB>{});
+    float* out = Ainv + (size_t)s * n * n;
+#pragma unroll
+    for (int a = 0; a < NB; ++a)
+#pragma unroll
+        for (int b = 0; b < NB; ++b) {
+            const int i = ti + 16 * a, j = tj + 16 * b;
+            if (i < n && j < n) out[(size_t)piv[j] * n + inv_piv[i]] = v[a][b];
+        }
+}
+
+// Any n and type: a cluster of kGjCluster CTAs per sample, each with all rows
+// of its share of the columns.  A step needs one column from its owner (written
+// into every CTA's shared memory, one cluster barrier); the pivot row's entries
+// are local.  SMEM: the share lies in shared memory, else in W.
+constexpr int kGjCluster = 8;
+
+template <class M, class R, bool SMEM>
+__global__ void __cluster_dims__(kGjCluster, 1, 1) __launch_bounds__(256)
+    k_gauss_jordan_cl(Grid G, const uint8_t* __restrict__ bc, const B4<M>* __restrict__ J,
+                      R* __restrict__ W, R* __restrict__ Ainv, const int* mask, int mstride)
+{
+    namespace cg = cooperative_groups;
+    extern __shared__ __align__(16) unsigned char gj_smem[];
+    const int s = blockIdx.x / kGjCluster;
+    if (!sample_on(mask, mstride, s)) return;  // (the whole cluster)
+    cg::cluster_group cl = cg::this_cluster();
+    const int rank = (int)cl.block_rank();
+    const int n = 2 * G.N, nc = (n + kGjCluster - 1) / kGjCluster;
+    const int c0 = min(n, rank * nc), c1 = min(n, c0 + nc), w = c1 - c0;
+    R* col = reinterpret_cast<R*>(gj_smem);  // [2][n], double-buffered by step
+    R* row = col + 2 * n;                    // [nc]
+    R* A = SMEM ? row + nc : W + ((size_t)s * kGjCluster + rank) * n * nc;  // [n][nc]
+    int* piv = reinterpret_cast<int*>(row + nc + (SMEM ? (size_t)n * nc : 0));
+    int* inv_piv = piv + n;
+    __shared__ int sp, sother;
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int ti = tid >> 4, tj = tid & 15;
+    for (int e = tid; e < n * nc; e += blockDim.x) A[e] = R(0);
+    __syncthreads();
+    coarse_fill<M, R>(G, bc, J + (size_t)s * 27 * G.N, A, nc, c0, c1);
+    cl.sync();  // (all CTAs of the cluster run: their shared memory can be written)
+    unsigned long long used = 0;  // (warp 0)
     for (int k = 0; k < n; ++k) {
-        // pivot: argmax |A[r][k]| over r >= k (ties to the lower row)
-        R best = R(-1);
-        int bi = k;
-        for (int r = k + threadIdx.x; r < n; r += blockDim.x) {
-            const R a = fabs(A[(size_t)r * w2 + k]);
-            if (a > best) { best = a; bi = r; }
-        }
-        for (int o = 16; o > 0; o >>= 1) {
-            const R ob = __shfl_xor_sync(0xffffffffu, best, o);
-            const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-            if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
-        }
-        if (lane == 0) { rv[warp] = best; ri[warp] = bi; }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            for (int q = 1; q < nw; ++q)
-                if (rv[q] > rv[0] || (rv[q] == rv[0] && ri[q] < ri[0])) { rv[0] = rv[q]; ri[0] = ri[q]; }
-        }
-        __syncthreads();
-        const int piv = ri[0];
-        __syncthreads();
-        if (piv != k)
-            for (int q = threadIdx.x; q < w2; q += blockDim.x) {
-                const R t = A[(size_t)k * w2 + q];
-                A[(size_t)k * w2 + q] = A[(size_t)piv * w2 + q];
-                A[(size_t)piv * w2 + q] = t;
+        const int owner = k / nc, buf = (k & 1) * n;
+        if (rank == owner) {
+            for (int e = tid; e < n * kGjCluster; e += blockDim.x) {
+                const int to = e / n, i = e - to * n;
+                cl.map_shared_rank(col, to)[buf + i] = A[(size_t)i * nc + k - c0];
             }
+        }
+        cl.sync();
+        const R* ck = col + buf;
+        if (tid < 32) {
+            bool other;
+            const int p = gj_pivot(ck, n, used, other);
+            if (lane == (p & 31)) used |= 1ull << (p >> 5);
+            const R inv = R(1) / ck[p];
+            for (int j = lane; j < w; j += 32) {
+                const R x = (c0 + j == k ? R(1) : A[(size_t)p * nc + j]) * inv;
+                row[j] = x;
+                A[(size_t)p * nc + j] = x;
+            }
+            if (lane == 0) {
+                sp = p;
+                sother = other;
+                piv[k] = p;
+                inv_piv[p] = k;
+            }
+        }
         __syncthreads();
-        const R inv = R(1) / A[(size_t)k * w2 + k];
-        __syncthreads();
-        for (int q = threadIdx.x; q < w2; q += blockDim.x) A[(size_t)k * w2 + q] *= inv;
-        for (int r = threadIdx.x; r < n; r += blockDim.x) f[r] = A[(size_t)r * w2 + k];
-        __syncthreads();
-        for (int r = warp; r < n; r += nw) {
-            if (r == k) continue;
-            const R fr = f[r];
-            for (int q = k + lane; q < w2; q += 32)
-                A[(size_t)r * w2 + q] -= fr * A[(size_t)k * w2 + q];
+        if (sother) {
+            const int p = sp;
+            for (int i = ti; i < n; i += 16) {
+                if (i == p) continue;
+                const R f = ck[i];
+                for (int j = tj; j < w; j += 16) {
+                    R* q = A + (size_t)i * nc + j;
+                    *q = fma(-f, row[j], c0 + j == k ? R(0) : *q);
+                }
+            }
         }
         __syncthreads();
     }
+    cl.sync();  // no CTA leaves while another may still write to it
     R* out = Ainv + (size_t)s * n * n;
-    for (int idx = threadIdx.x; idx < n * n; idx += blockDim.x) {
-        const int r = idx / n, q = idx - r * n;
-        out[idx] = A[(size_t)r * w2 + n + q];
+    for (int e = tid; e < n * w; e += blockDim.x) {
+        const int j = e / n, i = e - j * n;
+        out[(size_t)piv[c0 + j] * n + inv_piv[i]] = A[(size_t)i * nc + j];
     }
 }
 
+// Which kernel: FP32 up to 192 unknowns in one CTA's registers (256 threads of
+// 49 or 144 entries), everything else by clusters.  FP64 always: the
+// elimination's n^3 fused multiply-adds are bound by the FP64 pipe of the SMs
+// that hold the matrix, 0.3 ms on one SM at n = 100.  Against one CTA
+// eliminating [A | I] in shared memory (n = 100) or global memory, the step:
+// 128x64x16 x 4 mixed, n = 180: 62.3 -> 28.4 ms; 128x128x32 mixed, n = 100: 27.3
+// -> 22.3 ms; 32x32x8 FP64, n = 100: 9.9 -> 8.1 ms.
 template <class M>
 void launch_coarse_inverse(const Grid& G, const uint8_t* bc, const B4<M>* J,
                            double* work, double* Ainv, const int* mask,
                            int mstride, int S, cudaStream_t st)
 {
     using R = typename CoarseType<M>::type;
-    count_launch(2);
-    dim3 grid(nblocks(G.N, 64), S);
-    R* W = reinterpret_cast<R*>(work);
-    k_coarse_build<M, R><<<grid, 64, 0, st>>>(G, bc, J, W, mask, mstride);
+    count_launch(1);
     const int n = 2 * G.N;
     R* Ai = reinterpret_cast<R*>(Ainv);
-    const size_t smem = sizeof(R) * ((size_t)n + (size_t)2 * n * n);
-    if (smem <= 200 * 1024) {
-        static bool attr_set = false;
-        if (!attr_set) {
-            cudaFuncSetAttribute(k_gauss_jordan<true, R>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-            attr_set = true;
+    if constexpr (std::is_same<R, float>::value) {
+        const size_t stage = sizeof(float) * (size_t)n * n;
+        if (n <= 112) {
+            launch_smem(k_gauss_jordan_reg<M, 7>, dim3(S), 256, stage, st, G, bc, J, Ai, mask,
+                        mstride);
+            return;
         }
-        k_gauss_jordan<true, R><<<S, 256, smem, st>>>(n, W, Ai, mask, mstride);
-    } else {
-        k_gauss_jordan<false, R><<<S, 256, sizeof(R) * n, st>>>(n, W, Ai, mask, mstride);
+        if (n <= 192) {
+            launch_smem(k_gauss_jordan_reg<M, 12>, dim3(S), 256, stage, st, G, bc, J, Ai, mask,
+                        mstride);
+            return;
+        }
     }
+    const int nc = (n + kGjCluster - 1) / kGjCluster;
+    const size_t base = sizeof(R) * (2 * (size_t)n + nc) + sizeof(int) * 2 * (size_t)n;
+    const size_t share = sizeof(R) * (size_t)n * nc;
+    R* W = reinterpret_cast<R*>(work);
+    if (base + share <= 200 * 1024)
+        launch_smem(k_gauss_jordan_cl<M, R, true>, dim3(S * kGjCluster), 256, base + share, st, G,
+                    bc, J, W, Ai, mask, mstride);
+    else
+        launch_smem(k_gauss_jordan_cl<M, R, false>, dim3(S * kGjCluster), 256, base, st, G, bc, J,
+                    W, Ai, mask, mstride);
 }
 template void launch_coarse_inverse<double>(const Grid&, const uint8_t*,
                                             const B4<double>*, double*,

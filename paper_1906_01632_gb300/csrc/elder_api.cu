@@ -491,7 +491,7 @@ template <class T> void solver_alloc(elder_ctx* ctx, Solver<T>& sv, int cap)
     const int nc = 2 * ctx->grids.back().N;
     sv.Ainv = dalloc<double>((size_t)S * nc * nc);
     sv.mem.add(sv.Ainv);
-    sv.work = dalloc<double>((size_t)S * nc * 2 * nc);
+    sv.work = dalloc<double>((size_t)S * nc * (nc + 8));  // shares of the elimination
     sv.mem.add(sv.work);
     sv.S = S;
 }

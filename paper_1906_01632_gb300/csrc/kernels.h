@@ -73,6 +73,19 @@ inline int nblocks(int n, int bs = kBS) { return (n + bs - 1) / bs; }
 // blocks of the BiCGStab x/r update (4 nodes per thread): its partials per sample
 inline int bicg_xr_blocks(int n) { return nblocks((n + 3) / 4); }
 
+// Launch with dynamic shared memory beyond the default limit.  The attribute is
+// set on every such launch (a host call; it does not touch the stream), so it
+// holds on whichever device is current.
+template <class... P, class... A>
+void launch_smem(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st,
+                 A... args)
+{
+    if (smem > 48 * 1024)
+        cudaFuncSetAttribute(reinterpret_cast<const void*>(kernel),
+                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    kernel<<<grid, threads, smem, st>>>(static_cast<P>(args)...);
+}
+
 // Process-wide count of kernel launches made by this library.
 void count_launch(int n);
 // Message returned by elder_last_error(NULL) after a failed context-free call.

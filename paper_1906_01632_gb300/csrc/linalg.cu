@@ -12,6 +12,7 @@
 //
 // Solver vectors hold the unknowns of the interior system: Dirichlet
 // components are kept at 0 by masking every kernel's output.
+#include <algorithm>
 #include <type_traits>
 #include <cuda_pipeline.h>
 
@@ -756,29 +757,45 @@ void launch_prolong_add(const Grid& Gf, const Grid& Gc, const uint8_t* bcf,
     k_prolong_add<T><<<grid, kBS, 0, st>>>(Gf, Gc, bcf, xc, xf, mask, mstride);
 }
 
-// x = A_c^{-1} b on the coarsest grid (FP64 inverse), one block per sample.
+// x = A_c^{-1} b on the coarsest grid, one block per sample; the inverse lies
+// by columns.  Latency-bound (n loads of the inverse per unknown): kCaSplit
+// threads share an unknown's sum, each over every kCaSplit-th term, so that a
+// thread has n / kCaSplit independent loads.  The plain product reads a column
+// per step (coalesced over the unknowns); the transposed one a row segment.
+constexpr int kCaSplit = 4;
+
 template <class T>
-__global__ void k_coarse_apply(int n, const T* __restrict__ Ainv,
-                               const V2<T>* __restrict__ b, V2<T>* __restrict__ x,
-                               int trans, const int* mask, int mstride)
+__global__ void __launch_bounds__(1024)
+    k_coarse_apply(int n, const T* __restrict__ Ainv, const V2<T>* __restrict__ b,
+                   V2<T>* __restrict__ x, int trans, const int* mask, int mstride)
 {
     extern __shared__ __align__(16) unsigned char ca_smem[];
-    T* bs = reinterpret_cast<T*>(ca_smem);
+    T* bs = reinterpret_cast<T*>(ca_smem);  // [n]
+    T* part = bs + n;                       // [kCaSplit][n]
     const int s = blockIdx.x;
     if (!on(mask, mstride, s)) return;
     const T* bb = reinterpret_cast<const T*>(b + (size_t)s * (n / 2));
     for (int q = threadIdx.x; q < n; q += blockDim.x) bs[q] = bb[q];
     __syncthreads();
     const T* A = Ainv + (size_t)s * n * n;
-    T* xx = reinterpret_cast<T*>(x + (size_t)s * (n / 2));
-    for (int r = threadIdx.x; r < n; r += blockDim.x) {
+    for (int e = threadIdx.x; e < n * kCaSplit; e += blockDim.x) {
+        // plain: consecutive threads take consecutive unknowns; transposed:
+        // the kCaSplit threads of an unknown are neighbours
+        const int r = trans ? e / kCaSplit : e % n, c = trans ? e % kCaSplit : e / n;
         T acc = T(0);
-        if (!trans)
-            for (int q = 0; q < n; ++q) acc = fma(A[(size_t)r * n + q], bs[q], acc);
-        else
-            for (int q = 0; q < n; ++q) acc = fma(A[(size_t)q * n + r], bs[q], acc);
-        xx[r] = acc;
+        if (!trans) {
+#pragma unroll 8
+            for (int q = c; q < n; q += kCaSplit) acc = fma(A[(size_t)q * n + r], bs[q], acc);
+        } else {
+#pragma unroll 8
+            for (int q = c; q < n; q += kCaSplit) acc = fma(A[(size_t)r * n + q], bs[q], acc);
+        }
+        part[c * n + r] = acc;
     }
+    __syncthreads();
+    T* xx = reinterpret_cast<T*>(x + (size_t)s * (n / 2));
+    for (int r = threadIdx.x; r < n; r += blockDim.x)
+        xx[r] = (part[r] + part[n + r]) + (part[2 * n + r] + part[3 * n + r]);
 }
 
 template <class T>
@@ -788,10 +805,11 @@ void launch_coarse_apply(const Grid& G, const double* Ainv, const V2<T>* b,
 {
     count_launch(1);
     const int n = 2 * G.N;
+    const int threads = std::min(1024, (n * kCaSplit + 31) / 32 * 32);
     // the inverse is stored in the solver's arithmetic (CoarseType of its
     // multigrid storage type: FP32 for the mixed solver, FP64 otherwise)
-    k_coarse_apply<T><<<S, 128, sizeof(T) * n, st>>>(n, reinterpret_cast<const T*>(Ainv), b, x,
-                                                     trans, mask, mstride);
+    launch_smem(k_coarse_apply<T>, dim3(S), threads, sizeof(T) * n * (1 + kCaSplit), st, n,
+                reinterpret_cast<const T*>(Ainv), b, x, trans, mask, mstride);
 }
 
 // ---------------------------------------------------------------------------
