@@ -298,8 +298,8 @@ int elder_solve(elder_ctx* ctx, int S, const double* phi, const double* K,
  * (kind ELDER_SMOOTH_ILU; the transposed application uses the factors of
  * the untransposed operator).  Every kind needs no configuration: the
  * factors are formed for the call.  Computed in the context's multigrid
- * precision: FP64, or in ELDER_MIXED bfloat16 matrices and factors with
- * FP32 arithmetic and vectors.  r, z: [S][N][2] device (p, c interleaved);
+ * precision: FP64, or in ELDER_MIXED bfloat16 matrices and factors (the
+ * plain z-line application: FP32 line blocks) with FP32 arithmetic and vectors.  r, z: [S][N][2] device (p, c interleaved);
  * Dirichlet components of r are ignored, those of z are 0.  Used by the
  * parity tests of the smoothers. */
 int elder_smoother_apply(elder_ctx* ctx, int S, const double* phi, const double* K,
@@ -361,10 +361,15 @@ int elder_profile(elder_ctx* ctx, int on);
  *   SMOOTH  108 Mz + 10 T + 1    SMOOTH0  8 T + 1 (+ 8 Mz z-line)
  *   SPMV    108 T  + 6 T + 1     MGRES    108 Mz + 6 T + 1
  *   RESIDUAL 49 + 16 C/N         JACOBIAN 108 T + 108 Mz + 4 T + 17 + 16 C/N
+ * The finest level of the mixed solver under the z-line smoother stores no
+ * matrix (products from the state and the coefficients), there
+ *   SMOOTH0 16 T + 1    SPMV, MGRES 8 T + 2 T C/N + 1
+ *   JACOBIAN 36 T + 18 + 2 T C/N   SMOOTH 26 T + 2 T C/N + 2.
  * (the Jacobian writes the Krylov and the multigrid copies of J and the
  * inverse diagonal blocks; the residual reads p, c, c_old, phi, K and writes
  * R).  Flops: the FP64 residual counts 266 C/N + 75 of its factored face
- * form, the stencil products 216 + their vector terms.  Any output pointer
+ * form, the stencil products 216 + their vector terms, the matrix-free ones
+ * 512 C/N + 29.  Any output pointer
  * may be NULL.  Host outputs. */
 int elder_profile_read(const elder_ctx* ctx, int kernel_class,
                        int64_t* launches, double* ms, double* bytes,

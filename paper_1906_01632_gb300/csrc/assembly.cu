@@ -731,9 +731,7 @@ void launch_jacobian(const Grid& G, const Phys& ph, const uint8_t* bc,
         dim3 gin(nblocks(std::max(G.N, G.C)), S);
         k_jac_inputs<T><<<gin, kBS, 0, st>>>(G, ph, phi, K, p, c, cellT, nodeT, mask, mstride);
     } else if (inputs == 1) {  // the coefficients are converted already
-        count_launch(1);
-        k_node_inputs<T><<<dim3(nblocks(G.N), S), kBS, 0, st>>>(G, ph.rho0 * ph.g, p, c, nodeT,
-                                                                mask, mstride);
+        launch_node_inputs<T>(G, ph, p, c, nodeT, mask, mstride, S, st);
     }
     dim3 grid(nblocks(G.N, 128), S);
     // lumped storage volume per unit phi over dt: (h^3 / 8) / dt per cell corner
@@ -759,6 +757,85 @@ template void launch_jacobian<float, __nv_bfloat16>(const Grid&, const Phys&, co
                                                     B4<__nv_bfloat16>*, B4<float>*, V2<float>*,
                                                     V2<float>*, const int*, int, int,
                                                     cudaStream_t, int);
+
+template <class T>
+void launch_node_inputs(const Grid& G, const Phys& ph, const double* p, const double* c,
+                        V2<T>* nodeT, const int* mask, int mstride, int S, cudaStream_t st)
+{
+    count_launch(1);
+    k_node_inputs<T><<<dim3(nblocks(G.N), S), kBS, 0, st>>>(G, ph.rho0 * ph.g, p, c, nodeT, mask,
+                                                            mstride);
+}
+
+// The three blocks of a node's row that lie on its vertical line, as k_jacobian
+// forms them (the other 24 accumulators are dead code here), and the inverse
+// of the interior diagonal block.
+template <class T>
+__global__ void __launch_bounds__(128)
+    k_line_blocks(Grid G, PhysT<T> pt, GeomT<T> cg, const uint8_t* __restrict__ bc,
+                  const V2<T>* __restrict__ cellT, const V2<T>* __restrict__ nodeT,
+                  B4<T>* __restrict__ Dinv, B4<T>* __restrict__ Lz, B4<T>* __restrict__ Uz,
+                  T vscale, T* __restrict__ vs, const int* mask, int mstride)
+{
+    const int s = blockIdx.y;
+    if (blockIdx.x == 0 && s == 0 && threadIdx.x == 0) *vs = vscale;
+    if (!sample_on(mask, mstride, s)) return;
+    const int n = blockIdx.x * blockDim.x + threadIdx.x;
+    if (n >= G.N) return;
+    const size_t on = (size_t)s * G.N;
+    cellT += (size_t)s * G.C;
+    nodeT += on;
+    int i, j, k;
+    node_ijk(G, n, i, j, k);
+    T acc[27][4];
+#pragma unroll
+    for (int q = 0; q < 27; ++q)
+#pragma unroll
+        for (int r = 0; r < 4; ++r) acc[q][r] = T(0);
+    T phis = T(0);
+    jac_cell<T, -1, -1, -1>(G, pt, cg, i, j, k, cellT, nodeT, acc, phis);
+    jac_cell<T, 0, -1, -1>(G, pt, cg, i, j, k, cellT, nodeT, acc, phis);
+    jac_cell<T, -1, 0, -1>(G, pt, cg, i, j, k, cellT, nodeT, acc, phis);
+    jac_cell<T, 0, 0, -1>(G, pt, cg, i, j, k, cellT, nodeT, acc, phis);
+    jac_cell<T, -1, -1, 0>(G, pt, cg, i, j, k, cellT, nodeT, acc, phis);
+    jac_cell<T, 0, -1, 0>(G, pt, cg, i, j, k, cellT, nodeT, acc, phis);
+    jac_cell<T, -1, 0, 0>(G, pt, cg, i, j, k, cellT, nodeT, acc, phis);
+    jac_cell<T, 0, 0, 0>(G, pt, cg, i, j, k, cellT, nodeT, acc, phis);
+    const T vdt = phis * vscale;
+    T a = acc[13][0], b = acc[13][1] + vdt * pt.drho, d = acc[13][2];
+    T e = acc[13][3] + vdt * (pt.rho0 + T(2) * pt.drho * nodeT[n].c);
+    const uint8_t m = bc[n];
+    if (m & BC_P) { a = T(1); b = T(0); d = T(0); }
+    if (m & BC_C) { e = T(1); b = T(0); d = T(0); }
+    const T id = T(1) / (a * e - b * d);
+    Dinv[on + n] = B4<T>{e * id, -b * id, -d * id, a * id};
+    Lz[on + n] = B4<T>{acc[4][0], acc[4][1], acc[4][2], acc[4][3]};
+    Uz[on + n] = B4<T>{acc[22][0], acc[22][1], acc[22][2], acc[22][3]};
+}
+
+template <class T>
+void launch_line_blocks(const Grid& G, const Phys& ph, const uint8_t* bc, const V2<T>* cellT,
+                        const V2<T>* nodeT, B4<T>* Dinv, B4<T>* Lz, B4<T>* Uz, T* vs,
+                        const int* mask, int mstride, int S, cudaStream_t st)
+{
+    count_launch(1);
+    const CellGeom cgd = make_geom(G);
+    GeomT<T> cg;
+    for (int d = 0; d < 3; ++d) {
+        cg.ih[d] = T(cgd.ih[d]);
+        cg.area[d] = T(cgd.area[d]);
+    }
+    const PhysT<T> pt{T(ph.rho0), T(ph.drho), T(ph.g), T(ph.Dm)};
+    k_line_blocks<T><<<dim3(nblocks(G.N, 128), S), 128, 0, st>>>(
+        G, pt, cg, bc, cellT, nodeT, Dinv, Lz, Uz, T(0.125 * G.hx * G.hy * G.hz / ph.dt), vs,
+        mask, mstride);
+}
+template void launch_node_inputs<float>(const Grid&, const Phys&, const double*, const double*,
+                                        V2<float>*, const int*, int, int, cudaStream_t);
+template void launch_line_blocks<float>(const Grid&, const Phys&, const uint8_t*,
+                                        const V2<float>*, const V2<float>*, B4<float>*,
+                                        B4<float>*, B4<float>*, float*, const int*, int, int,
+                                        cudaStream_t);
 
 // ---------------------------------------------------------------------------
 // hierarchy: state injection, cell averaging, block-diagonal inverse

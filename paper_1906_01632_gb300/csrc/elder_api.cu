@@ -143,6 +143,14 @@ struct SolverBase {
 template <class T> struct Solver : SolverBase {
     int S = 0;
     using M = typename MgType<T>::type;
+    // The mixed solver's finest level needs no stored matrix (mf): products
+    // by launch_mf_apply, line blocks Lz, Uz and |scv| / dt (vs) from
+    // launch_line_blocks.  J0 and Jm[0] are then allocated by the first call
+    // that needs the rows (reserve_rows); mf_now: the assembly in use has none.
+    bool mf = false, mf_now = false;
+    B4<T> *Lz = nullptr, *Uz = nullptr;
+    T* vs = nullptr;
+    Phys phys{};                   // of the assembly in use
     B4<T>* J0 = nullptr;           // level-0 Krylov operator (T)
     std::vector<B4<M>*> Jm;        // multigrid matrices per level (M)
     std::vector<B4<T>*> Dinv;      // inverse interior diagonal blocks per level
@@ -294,7 +302,7 @@ double configured_omega(const elder_config& cf)
     return cf.smoother == ELDER_SMOOTH_ZLINE ? cf.omega_line : cf.omega;
 }
 
-double model_bytes(int cls, int T, int Mz, const Grid& G, int line)
+double model_bytes(int cls, int T, int Mz, const Grid& G, int line, bool mf)
 {
     // T: bytes of a vector / Dinv entry; Mz: bytes of a stored matrix entry
     // (for the Jacobian class: Mz of the multigrid copy, T of the Krylov copy
@@ -306,8 +314,24 @@ double model_bytes(int cls, int T, int Mz, const Grid& G, int line)
     // scratch vector written, read and written again, x_out, bc twice).
     // line (JACOBIAN): bit 0 with the line factorisation, bit 1 with the ILU
     // factorisation (J, Dinv and bc read, the factors written).
+    // mf: the mixed solver's finest level, whose operator is not stored
+    // (products from the state (p', c) and the coefficients (phi, K/mu), line
+    // blocks in T).
     const double cells_per_node = (double)G.C / G.N;
     const int Td = T ? T : Mz;
+    const double mf_inputs = 2 * T + 2 * T * cells_per_node;
+    if (mf) {
+        switch (cls) {
+        case ELDER_K_SMOOTH: return mf_inputs + (6 + 4 + 4 + 4 + 6) * T + 2;
+        case ELDER_K_SMOOTH0: return (4 + 4 + 4 + 2 + 2) * T + 1;  // zMi, zC, L, b, xo, bc
+        case ELDER_K_SPMV: return mf_inputs + (2 + 2 + 2) * T + 1;   // x, y, a, bc
+        case ELDER_K_MGRES: return mf_inputs + (2 + 2 + 2) * T + 1;  // x, b, r, bc
+        case ELDER_K_JACOBIAN:
+            // node inputs; Dinv, L, U written; line factors: they and bc
+            // read, zMi, zC written
+            return 16 + 2 * T + mf_inputs + 1 + 12 * T + (12 + 8) * T + 1;
+        }
+    }
     switch (cls) {
     case ELDER_K_SMOOTH: return 108 * Mz + (4 + 2 + 2 + 2) * T + 1;  // J, Dinv, b, x, xo, bc
     case ELDER_K_SMOOTH0:
@@ -327,9 +351,14 @@ double model_bytes(int cls, int T, int Mz, const Grid& G, int line)
     return 0.0;
 }
 
-double model_flops(int cls, const Grid& G)
+double model_flops(int cls, const Grid& G, bool mf)
 {
     const double cells_per_node = (double)G.C / G.N;
+    // matrix-free product, per cell: row sums 68, passes across the rows and
+    // differences 128, 12 faces of 25 with their corner sums (+4 on vertical
+    // edges): 512; per node 6 corner sums of 3 values and 11 for storage: 29
+    if (mf && (cls == ELDER_K_SPMV || cls == ELDER_K_MGRES))
+        return 512 * cells_per_node + 29;
     switch (cls) {
     case ELDER_K_SMOOTH: return 216 + 8 + 4 + 4;
     case ELDER_K_SMOOTH0: return 8 + 2;
@@ -372,7 +401,7 @@ int prof_begin(elder_ctx* ctx, cudaStream_t st)
 // variant: for SMOOTH0 -1 = by the smoother in use, 2 = the factored z-line
 // sweep; for JACOBIAN 1 = with the line factorisation
 void prof_end(elder_ctx* ctx, int idx, int cls, const Grid& G, int T, int Mz, int samples,
-              cudaStream_t st, int variant = -1)
+              cudaStream_t st, int variant = -1, bool mf = false)
 {
     if (idx < 0) return;
     ProfRec& r = ctx->prof.pending[idx];
@@ -380,8 +409,8 @@ void prof_end(elder_ctx* ctx, int idx, int cls, const Grid& G, int T, int Mz, in
     r.cls = cls;
     int line = ctx->smoother_now == ELDER_SMOOTH_ZLINE && G.nz + 1 <= kMaxLine ? 1 : 0;
     if (variant >= 0) line = variant;
-    r.bytes = model_bytes(cls, T, Mz, G, line) * G.N * samples;
-    r.flops = model_flops(cls, G) * G.N * samples;
+    r.bytes = model_bytes(cls, T, Mz, G, line, mf) * G.N * samples;
+    r.flops = model_flops(cls, G, mf) * G.N * samples;
 }
 
 // after a stream synchronisation: accumulate and recycle the events
@@ -442,12 +471,30 @@ template <class T> void solver_alloc(elder_ctx* ctx, Solver<T>& sv, int cap)
     }
     const int S = cap;
     const int L = (int)ctx->grids.size();
+    // a matrix-free finest level: in FP32, under the z-line smoother (the
+    // others sweep with the rows) and above a coarser level (the coarsest is
+    // inverted from its rows)
+    sv.mf = std::is_same<T, float>::value && L > 1 && ctx->cfg.smoother == ELDER_SMOOTH_ZLINE &&
+            ctx->grids[0].nz + 1 <= kMaxLine;
+    if (sv.mf) {
+        const size_t n0 = (size_t)S * ctx->grids[0].N;
+        for (B4<T>** q : {&sv.Lz, &sv.Uz}) {
+            *q = dalloc<B4<T>>(n0);
+            sv.mem.add(*q);
+        }
+        sv.vs = dalloc<T>(1);
+        sv.mem.add(sv.vs);
+    }
     for (int l = 0; l < L; ++l) {
         const Grid& G = ctx->grids[l];
         const size_t nN = (size_t)S * G.N;
-        sv.Jm.push_back(dalloc<B4<typename Solver<T>::M>>(nN * 27));
-        sv.mem.add(sv.Jm.back());
-        if (l == 0) {
+        if (l == 0 && sv.mf) {
+            sv.Jm.push_back(nullptr);
+        } else {
+            sv.Jm.push_back(dalloc<B4<typename Solver<T>::M>>(nN * 27));
+            sv.mem.add(sv.Jm.back());
+        }
+        if (l == 0 && !sv.mf) {
             if (std::is_same<T, typename Solver<T>::M>::value) {
                 sv.J0 = reinterpret_cast<B4<T>*>(sv.Jm[0]);  // one array serves both
             } else {
@@ -496,16 +543,32 @@ template <class T> void solver_alloc(elder_ctx* ctx, Solver<T>& sv, int cap)
     sv.S = S;
 }
 
+// Room for the finest level's rows of a matrix-free solver.
+template <class T> void reserve_rows(elder_ctx* ctx, Solver<T>& sv)
+{
+    if (sv.J0) return;
+    const size_t n = (size_t)sv.S * ctx->grids[0].N * 27;
+    sv.Jm[0] = dalloc<B4<typename Solver<T>::M>>(n);
+    sv.mem.add(sv.Jm[0]);
+    sv.J0 = dalloc<B4<T>>(n);
+    sv.mem.add(sv.J0);
+}
+
 // Re-discretised Jacobians on every level (Section 5.1): level 0 at the
 // current iterate, coarser levels at the injected state with the averaged
 // coefficients; then the block-diagonal inverses and the coarse inverse.
+// rows: the finest level's rows are needed (transposed solves, the other
+// smoothers) also where the solver can do without.
 template <class T>
 void assemble(elder_ctx* ctx, Solver<T>& sv, int S, const double* phi0,
               const double* K0, const double* p0, const double* c0,
               const Phys& ph, const int* mask, int mstride, int n_active,
-              cudaStream_t st)
+              cudaStream_t st, bool rows = false)
 {
     const int L = (int)ctx->grids.size();
+    if (rows) reserve_rows<T>(ctx, sv);
+    sv.mf_now = sv.mf && !rows;
+    sv.phys = ph;
     for (int l = 0; l < L; ++l) {
         const Grid& G = ctx->grids[l];
         const double* phi = l == 0 ? phi0 : ctx->phi[l];
@@ -522,6 +585,18 @@ void assemble(elder_ctx* ctx, Solver<T>& sv, int S, const double* phi0,
         }
         const int pi = prof_begin(ctx, st);
         using M = typename Solver<T>::M;
+        if constexpr (std::is_same<T, float>::value) {
+            if (l == 0 && sv.mf_now) {
+                launch_node_inputs<T>(G, ph, p, c, nodeT, mask, mstride, S, st);
+                launch_line_blocks<T>(G, ph, ctx->bc[0], cellT, nodeT, sv.Dinv[0], sv.Lz, sv.Uz,
+                                      sv.vs, mask, mstride, S, st);
+                launch_zline_factor<T, T>(G, sv.Lz, sv.Uz, (size_t)G.N, sv.Dinv[0], ctx->bc[0],
+                                          sv.zMi[0], sv.zC[0], mask, mstride, S, st);
+                prof_end(ctx, pi, ELDER_K_JACOBIAN, G, (int)sizeof(T), (int)sizeof(M), n_active,
+                         st, 1, true);
+                continue;
+            }
+        }
         B4<T>* JT = (l == 0 && !std::is_same<T, M>::value) ? sv.J0 : nullptr;
         // the cell inputs of every level were converted once for the step
         // (average_coefficients); the coarse node inputs came with the
@@ -530,8 +605,10 @@ void assemble(elder_ctx* ctx, Solver<T>& sv, int S, const double* phi0,
                               nodeT, mask, mstride, S, st, l == 0 ? 1 : 2);
         // the vertical lines' block-LU factors for the z-line sweeps
         if (sv.zMi[l])
-            launch_zline_factor<T, M>(G, sv.Jm[l], sv.Dinv[l], ctx->bc[l], sv.zMi[l], sv.zC[l],
-                                      mask, mstride, S, st);
+            launch_zline_factor<T, M>(G, sv.Jm[l] + slot27(0, 0, -1) * (size_t)G.N,
+                                      sv.Jm[l] + slot27(0, 0, 1) * (size_t)G.N, 27 * (size_t)G.N,
+                                      sv.Dinv[l], ctx->bc[l], sv.zMi[l], sv.zC[l], mask, mstride,
+                                      S, st);
         // the multicolour ILU factors for the ILU sweeps
         if (sv.F[l])
             launch_ilu_factor<T, M>(G, sv.Jm[l], sv.Dinv[l], ctx->bc[l], sv.F[l], sv.Fd[l],
@@ -562,6 +639,31 @@ void average_coefficients(elder_ctx* ctx, int S, const double* phi0,
                               l == 0 ? K0 : ctx->K[l], reinterpret_cast<V2<T>*>(ctx->jc[l]),
                               S, st);
     CKL();
+}
+
+// y = A x on the finest level (mode, a, partial as launch_spmv).
+template <class T>
+void apply_finest(elder_ctx* ctx, Solver<T>& sv, const V2<T>* x, V2<T>* y, int trans, int mode,
+                  const V2<T>* a, double* partial, const int* mask, int mstride, int S,
+                  cudaStream_t st, int bs = kBS)
+{
+    const Grid& G = ctx->grids[0];
+    if constexpr (std::is_same<T, float>::value) {
+        if (sv.mf_now) {
+            launch_mf_apply(G, sv.phys, ctx->bc[0], reinterpret_cast<const V2<T>*>(ctx->jc[0]),
+                            reinterpret_cast<const V2<T>*>(ctx->jn[0]), x, y, mode, a, partial,
+                            sv.vs, mask, mstride, S, st);
+            return;
+        }
+    }
+    launch_spmv<T>(G, sv.J0, ctx->bc[0], x, y, trans, mode, a, partial, mask, mstride, S, st, bs);
+}
+
+// Partials per sample that apply_finest leaves for its inner products.
+template <class T> int finest_partials(elder_ctx* ctx, const Solver<T>& sv, int S)
+{
+    const Grid& G = ctx->grids[0];
+    return sv.mf_now ? mf_blocks(G, S) : nblocks(G.N, 32);
 }
 
 // One V-cycle: out = M b on level l (masked by the Krylov flags).
@@ -597,31 +699,52 @@ void vcycle(elder_ctx* ctx, Solver<T>& sv, int l, const V2<T>* b, V2<T>* out,
     // the ILU sweeps keep their triangular solves in the level's residual
     // vector (free until the restriction's residual is formed)
     const bool ilu = ctx->smoother_now == ELDER_SMOOTH_ILU && sv.F[l];
+    const bool mf = l == 0 && sv.mf_now;
+    // r = b - A x
+    auto residual = [&](const V2<T>* xin, int spc) {
+        if constexpr (std::is_same<T, float>::value) {
+            if (mf) {
+                launch_mf_apply(G, sv.phys, ctx->bc[0], reinterpret_cast<const V2<T>*>(ctx->jc[0]),
+                                reinterpret_cast<const V2<T>*>(ctx->jn[0]), xin, sv.mr[0], 3, b,
+                                nullptr, sv.vs, mask, KSTRIDE, S, st);
+                return;
+            }
+        }
+        launch_mg_residual<T, M>(G, sv.Jm[l], ctx->bc[l], b, xin, sv.mr[l], trans, mask, KSTRIDE,
+                                 S, st, bs_mr, spc);
+    };
+    // the substitution of a factored z-line sweep
+    auto line_solve = [&](const V2<T>* rin, const V2<T>* xin, V2<T>* xout, int mode) {
+        if (mf)
+            launch_zline_apply<T, T>(G, sv.Lz, (size_t)G.N, sv.zMi[l], sv.zC[l], ctx->bc[l], rin,
+                                     xin, xout, ctx->omega_now, mask, KSTRIDE, S, st, mode, bs_zl,
+                                     spc_zl);
+        else
+            launch_zline_apply<T, M>(G, sv.Jm[l] + slot27(0, 0, -1) * (size_t)G.N,
+                                     27 * (size_t)G.N, sv.zMi[l], sv.zC[l], ctx->bc[l], rin, xin,
+                                     xout, ctx->omega_now, mask, KSTRIDE, S, st, mode, bs_zl,
+                                     spc_zl);
+    };
     auto sweep = [&](const V2<T>* xin, V2<T>* xout) {
         if (ilu && xin == nullptr) {
             launch_ilu_apply<T, M>(G, sv.F[l], sv.Fd[l], ctx->bc[l], b, sv.mr[l], nullptr, xout,
                                    ctx->omega_now, trans, 1, mask, KSTRIDE, S, st);
         } else if (ilu) {
-            launch_mg_residual<T, M>(G, sv.Jm[l], ctx->bc[l], b, xin, sv.mr[l], trans, mask,
-                                     KSTRIDE, S, st, bs_mr, spc_mr);
+            residual(xin, spc_mr);
             launch_ilu_apply<T, M>(G, sv.F[l], sv.Fd[l], ctx->bc[l], sv.mr[l], sv.mr[l], xin,
                                    xout, ctx->omega_now, trans, 2, mask, KSTRIDE, S, st);
         } else if (fact && xin == nullptr) {
-            launch_zline_apply<T, M>(G, sv.Jm[l], sv.zMi[l], sv.zC[l], ctx->bc[l], b, nullptr,
-                                     xout, ctx->omega_now, mask, KSTRIDE, S, st, 1, bs_zl, spc_zl);
+            line_solve(b, nullptr, xout, 1);
         } else if (fact) {
-            launch_mg_residual<T, M>(G, sv.Jm[l], ctx->bc[l], b, xin, sv.mr[l], trans, mask,
-                                     KSTRIDE, S, st, bs_mr, spc_mr);
-            launch_zline_apply<T, M>(G, sv.Jm[l], sv.zMi[l], sv.zC[l], ctx->bc[l], sv.mr[l], xin,
-                                     xout, ctx->omega_now, mask, KSTRIDE, S, st, 2, bs_zl, spc_zl);
+            residual(xin, spc_mr);
+            line_solve(sv.mr[l], xin, xout, 2);
         } else if (line && xin == nullptr) {
             launch_smooth_zline<T, M>(G, sv.Jm[l], sv.Dinv[l], ctx->bc[l], b, xin, xout,
                                       ctx->omega_now, trans, mask, KSTRIDE, S, st, 1);
         } else if (line) {
             // residual at full stream rate into the level's residual vector
             // (free once the restriction has been made), then the line solves
-            launch_mg_residual<T, M>(G, sv.Jm[l], ctx->bc[l], b, xin, sv.mr[l], trans, mask,
-                                     KSTRIDE, S, st, bs_mr);
+            residual(xin, 1);
             launch_smooth_zline<T, M>(G, sv.Jm[l], sv.Dinv[l], ctx->bc[l], sv.mr[l], xin, xout,
                                       ctx->omega_now, trans, mask, KSTRIDE, S, st, 2);
         } else
@@ -631,17 +754,16 @@ void vcycle(elder_ctx* ctx, Solver<T>& sv, int l, const V2<T>* b, V2<T>* out,
     int pi = prof_begin(ctx, st);
     sweep(nullptr, cur);
     prof_end(ctx, pi, ELDER_K_SMOOTH0, G, sizeof(T), sizeof(M), na, st,
-             ilu ? 3 : (fact ? 2 : -1));
+             ilu ? 3 : (fact ? 2 : -1), mf);
     for (int q = 1; q < nu1; ++q) {
         pi = prof_begin(ctx, st);
         sweep(cur, oth);
-        prof_end(ctx, pi, ELDER_K_SMOOTH, G, sizeof(T), sizeof(M), na, st);
+        prof_end(ctx, pi, ELDER_K_SMOOTH, G, sizeof(T), sizeof(M), na, st, -1, mf);
         std::swap(cur, oth);
     }
     pi = prof_begin(ctx, st);
-    launch_mg_residual<T, M>(G, sv.Jm[l], ctx->bc[l], b, cur, sv.mr[l], trans, mask, KSTRIDE, S,
-                             st, bs_mr, spc_mr);
-    prof_end(ctx, pi, ELDER_K_MGRES, G, sizeof(T), sizeof(M), na, st);
+    residual(cur, spc_mr);
+    prof_end(ctx, pi, ELDER_K_MGRES, G, sizeof(T), sizeof(M), na, st, -1, mf);
     launch_restrict<T>(G, ctx->grids[l + 1], ctx->bc[l + 1], sv.mr[l], sv.mb[l + 1], mask,
                        KSTRIDE, S, st);
     vcycle<T>(ctx, sv, l + 1, sv.mb[l + 1], sv.mx[l + 1], trans, S, st);
@@ -650,7 +772,7 @@ void vcycle(elder_ctx* ctx, Solver<T>& sv, int l, const V2<T>* b, V2<T>* out,
     for (int q = 0; q < nu2; ++q) {
         pi = prof_begin(ctx, st);
         sweep(cur, oth);
-        prof_end(ctx, pi, ELDER_K_SMOOTH, G, sizeof(T), sizeof(M), na, st);
+        prof_end(ctx, pi, ELDER_K_SMOOTH, G, sizeof(T), sizeof(M), na, st, -1, mf);
         std::swap(cur, oth);
     }
     if (cur != out) CK(cudaMemcpyAsync(out, cur, sizeof(V2<T>) * (size_t)S * G.N,
@@ -659,8 +781,8 @@ void vcycle(elder_ctx* ctx, Solver<T>& sv, int l, const V2<T>* b, V2<T>* out,
 
 // Autotuner: threads per block of the three J-streaming kernel classes,
 // chosen once per context and precision by timing every candidate (CUDA
-// events, 3 launches after a warm-up) on the first assembled level-0
-// operator of a step with all S samples active.
+// events, 3 launches after a warm-up) on the finest stored
+// operator of a step's first assembly with all S samples active.
 template <class T>
 void autotune(elder_ctx* ctx, Solver<T>& sv, int S, cudaStream_t st)
 {
@@ -672,28 +794,33 @@ void autotune(elder_ctx* ctx, Solver<T>& sv, int S, cudaStream_t st)
         return;
     }
     using M = typename Solver<T>::M;
-    const Grid& G = ctx->grids[0];
+    // on the finest level with a stored matrix (the products of a matrix-free
+    // level choose their tiles by the grid)
+    const int lt = sv.mf_now ? 1 : 0;
+    const Grid& G = ctx->grids[lt];
+    const uint8_t* bc = ctx->bc[lt];
     const size_t nv = (size_t)S * G.N;
-    CK(cudaMemsetAsync(sv.mb[0], 0, sizeof(V2<T>) * nv, st));
-    CK(cudaMemsetAsync(sv.mx[0], 0, sizeof(V2<T>) * nv, st));
+    CK(cudaMemsetAsync(sv.mb[lt], 0, sizeof(V2<T>) * nv, st));
+    CK(cudaMemsetAsync(sv.mx[lt], 0, sizeof(V2<T>) * nv, st));
     cudaEvent_t e0, e1;
     CK(cudaEventCreate(&e0));
     CK(cudaEventCreate(&e1));
     const int cand[3] = {kMinBS, kBS, kMaxBS};
     const int cls[3] = {ELDER_K_SMOOTH, ELDER_K_SPMV, ELDER_K_MGRES};
     for (int c = 0; c < 3; ++c) {
+        if (c == 1 && sv.mf_now) continue;
         float best = 1e30f;
         for (int q = 0; q < 3; ++q) {
             auto run = [&]() {
                 if (c == 0)
-                    launch_smooth<T, M>(G, sv.Jm[0], sv.Dinv[0], ctx->bc[0], sv.mb[0], sv.mx[0],
-                                        sv.mx2[0], ctx->cfg.omega, 0, nullptr, 0, S, st, cand[q]);
+                    launch_smooth<T, M>(G, sv.Jm[lt], sv.Dinv[lt], bc, sv.mb[lt], sv.mx[lt],
+                                        sv.mx2[lt], ctx->cfg.omega, 0, nullptr, 0, S, st, cand[q]);
                 else if (c == 1)
-                    launch_spmv<T>(G, sv.J0, ctx->bc[0], sv.mx[0], sv.mx2[0], 0, 0, nullptr,
+                    launch_spmv<T>(G, sv.J0, bc, sv.mx[lt], sv.mx2[lt], 0, 0, nullptr,
                                    nullptr, nullptr, 0, S, st, cand[q]);
                 else
-                    launch_mg_residual<T, M>(G, sv.Jm[0], ctx->bc[0], sv.mb[0], sv.mx[0],
-                                             sv.mx2[0], 0, nullptr, 0, S, st, cand[q]);
+                    launch_mg_residual<T, M>(G, sv.Jm[lt], bc, sv.mb[lt], sv.mx[lt],
+                                             sv.mx2[lt], 0, nullptr, 0, S, st, cand[q]);
             };
             run();
             CK(cudaEventRecord(e0, st));
@@ -713,7 +840,7 @@ void autotune(elder_ctx* ctx, Solver<T>& sv, int S, cudaStream_t st)
     // the factored z-line sweep from x = 0 (the default V(1,0) cycle's only
     // sweep); two samples per CTA give a thread two independent stencil rows
     // or line recursions
-    if (sv.zMi[0] && G.nz + 1 <= kMaxLine) {
+    if (sv.zMi[lt] && G.nz + 1 <= kMaxLine) {
         const int bsm[3] = {kMinBS, kBS, kMaxBS}, bsz[3] = {64, 128, 256};
         for (int c = 0; c < 2; ++c) {
             float best = 1e30f;
@@ -721,11 +848,12 @@ void autotune(elder_ctx* ctx, Solver<T>& sv, int S, cudaStream_t st)
                 const int bsq = c == 0 ? bsm[q % 3] : bsz[q % 3], spq = 1 + q / 3;
                 auto run = [&]() {
                     if (c == 0)
-                        launch_mg_residual<T, M>(G, sv.Jm[0], ctx->bc[0], sv.mb[0], sv.mx[0],
-                                                 sv.mx2[0], 0, nullptr, 0, S, st, bsq, spq);
+                        launch_mg_residual<T, M>(G, sv.Jm[lt], bc, sv.mb[lt], sv.mx[lt],
+                                                 sv.mx2[lt], 0, nullptr, 0, S, st, bsq, spq);
                     else
-                        launch_zline_apply<T, M>(G, sv.Jm[0], sv.zMi[0], sv.zC[0], ctx->bc[0],
-                                                 sv.mb[0], nullptr, sv.mx2[0], 1.0, nullptr, 0, S,
+                        launch_zline_apply<T, M>(G, sv.Jm[lt] + slot27(0, 0, -1) * (size_t)G.N,
+                                                 27 * (size_t)G.N, sv.zMi[lt], sv.zC[lt], bc,
+                                                 sv.mb[lt], nullptr, sv.mx2[lt], 1.0, nullptr, 0, S,
                                                  st, 1, bsq, spq);
                 };
                 run();
@@ -757,22 +885,22 @@ void bicg_iteration(elder_ctx* ctx, Solver<T>& sv, int trans, double rtol, int m
 {
     const Grid& G = ctx->grids[0];
     const int bs_mv = ctx->bs[ELDER_K_SPMV];
-    const int nb_mv = nblocks(G.N, 32);  // per-warp partials of the stencil products
+    const int nb_mv = finest_partials<T>(ctx, sv, S);  // partials of the products
     KScal* ks = ctx->ks;
     const int* mask = &ks[0].active;
     launch_bicg_p<T>(G, sv.r, sv.v, sv.p, ks, S, st);
     vcycle<T>(ctx, sv, 0, sv.p, sv.ph, trans, S, st);
     int pi = prof_begin(ctx, st);
-    launch_spmv<T>(G, sv.J0, ctx->bc[0], sv.ph, sv.v, trans, 1, sv.rh, ctx->partial, mask,
-                   KSTRIDE, S, st, bs_mv);
-    prof_end(ctx, pi, ELDER_K_SPMV, G, sizeof(T), sizeof(T), ctx->n_active_k, st);
+    apply_finest<T>(ctx, sv, sv.ph, sv.v, trans, 1, sv.rh, ctx->partial, mask, KSTRIDE, S, st,
+                    bs_mv);
+    prof_end(ctx, pi, ELDER_K_SPMV, G, sizeof(T), sizeof(T), ctx->n_active_k, st, -1, sv.mf_now);
     launch_bicg_finalize(1, ctx->partial, nb_mv, ks, rtol, maxit, S, st);
     launch_bicg_s<T>(G, sv.r, sv.v, sv.s, nullptr, ks, S, st);
     vcycle<T>(ctx, sv, 0, sv.s, sv.sh, trans, S, st);
     pi = prof_begin(ctx, st);
-    launch_spmv<T>(G, sv.J0, ctx->bc[0], sv.sh, sv.t, trans, 2, sv.s, ctx->partial, mask,
-                   KSTRIDE, S, st, bs_mv);
-    prof_end(ctx, pi, ELDER_K_SPMV, G, sizeof(T), sizeof(T), ctx->n_active_k, st);
+    apply_finest<T>(ctx, sv, sv.sh, sv.t, trans, 2, sv.s, ctx->partial, mask, KSTRIDE, S, st,
+                    bs_mv);
+    prof_end(ctx, pi, ELDER_K_SPMV, G, sizeof(T), sizeof(T), ctx->n_active_k, st, -1, sv.mf_now);
     launch_bicg_finalize(2, ctx->partial, nb_mv, ks, rtol, maxit, S, st);
     launch_bicg_xr<T>(G, sv.ph, sv.sh, sv.s, sv.t, sv.rh, sv.x, sv.r, ctx->partial, ks, S, st);
     launch_bicg_finalize(3, ctx->partial, bicg_xr_blocks(G.N), ks, rtol, maxit, S, st);
@@ -1476,7 +1604,7 @@ int solve_impl(elder_ctx* ctx, int S, const double* phi, const double* K, const 
     const Phys ph = make_phys(ctx->cfg, dt);
     const size_t nN = (size_t)S * G.N;
     average_coefficients<T>(ctx, S, phi, K, st);
-    assemble<T>(ctx, sv, S, phi, K, p, c, ph, nullptr, 0, S, st);
+    assemble<T>(ctx, sv, S, phi, K, p, c, ph, nullptr, 0, S, st, trans != 0);
     const V2<double>* rhs2 = reinterpret_cast<const V2<double>*>(rhs);
     V2<double>* x2 = reinterpret_cast<V2<double>*>(x);
     // rhs in solver precision
@@ -1491,8 +1619,8 @@ int solve_impl(elder_ctx* ctx, int S, const double* phi, const double* K, const 
     // (x_D is kept in sv.xd: the multigrid vectors are overwritten by the solve)
     if (!trans) {
         launch_axpy_mask<T>(G, ctx->bc[0], bT, sv.xd, 1.0, 0, S, st);     // xd = b on D
-        launch_spmv<T>(G, sv.J0, ctx->bc[0], sv.xd, sv.mx2[0], 0, 0, nullptr, nullptr,
-                       nullptr, 0, S, st);                                 // J x_D (interior)
+        apply_finest<T>(ctx, sv, sv.xd, sv.mx2[0], 0, 0, nullptr, nullptr, nullptr, 0, S,
+                        st);                                               // J x_D (interior)
         launch_axpy_mask<T>(G, ctx->bc[0], sv.mx2[0], bT, -1.0, 2, S, st);
     }
     bicgstab<T>(ctx, sv, trans, rtol, ctx->cfg.lin_maxit, nullptr, S, st);
@@ -1539,7 +1667,8 @@ void smoother_apply_impl(elder_ctx* ctx, int S, const double* phi, const double*
     const Grid& G = ctx->grids[0];
     const size_t nN = (size_t)S * G.N;
     average_coefficients<T>(ctx, S, phi, K, st);
-    assemble<T>(ctx, sv, S, phi, K, p, c, make_phys(ctx->cfg, dt), nullptr, 0, S, st);
+    assemble<T>(ctx, sv, S, phi, K, p, c, make_phys(ctx->cfg, dt), nullptr, 0, S, st,
+                kind != ELDER_SMOOTH_ZLINE || trans);
     V2<T>* bT = sv.b;
     if (std::is_same<T, double>::value)
         CK(cudaMemcpyAsync(bT, r, sizeof(double) * 2 * nN, cudaMemcpyDeviceToDevice, st));
@@ -1550,9 +1679,13 @@ void smoother_apply_impl(elder_ctx* ctx, int S, const double* phi, const double*
         launch_smooth<T, M>(G, sv.Jm[0], sv.Dinv[0], ctx->bc[0], bT, nullptr, sv.x, 1.0, trans,
                             nullptr, 0, S, st, kBS);
     } else if (kind == ELDER_SMOOTH_ZLINE) {
-        if (!trans && sv.zMi[0])
-            launch_zline_apply<T, M>(G, sv.Jm[0], sv.zMi[0], sv.zC[0], ctx->bc[0], bT, nullptr,
-                                     sv.x, 1.0, nullptr, 0, S, st, 1);
+        if (sv.mf_now)
+            launch_zline_apply<T, T>(G, sv.Lz, (size_t)G.N, sv.zMi[0], sv.zC[0], ctx->bc[0], bT,
+                                     nullptr, sv.x, 1.0, nullptr, 0, S, st, 1);
+        else if (!trans && sv.zMi[0])
+            launch_zline_apply<T, M>(G, sv.Jm[0] + slot27(0, 0, -1) * (size_t)G.N,
+                                     27 * (size_t)G.N, sv.zMi[0], sv.zC[0], ctx->bc[0], bT,
+                                     nullptr, sv.x, 1.0, nullptr, 0, S, st, 1);
         else
             launch_smooth_zline<T, M>(G, sv.Jm[0], sv.Dinv[0], ctx->bc[0], bT, nullptr, sv.x,
                                       1.0, trans, nullptr, 0, S, st, 1);

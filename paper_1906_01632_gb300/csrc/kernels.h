@@ -110,6 +110,17 @@ void launch_jacobian(const Grid& G, const Phys& ph, const uint8_t* bc,
                      const double* c, B4<T>* JT, B4<M>* JM, B4<T>* Dinv, V2<T>* cellT,
                      V2<T>* nodeT, const int* mask, int mask_stride, int S, cudaStream_t st,
                      int inputs = 0);
+// (p - rho0 g (Lz - z), c) in T for every node of the active samples
+template <class T>
+void launch_node_inputs(const Grid& G, const Phys& ph, const double* p, const double* c,
+                        V2<T>* nodeT, const int* mask, int mstride, int S, cudaStream_t st);
+// The blocks of the Jacobian along the vertical grid lines: inverse interior
+// diagonal blocks, and those of the offsets (0, 0, -1) and (0, 0, +1) [S][N];
+// *vs receives |scv| / dt for launch_mf_apply.
+template <class T>
+void launch_line_blocks(const Grid& G, const Phys& ph, const uint8_t* bc, const V2<T>* cellT,
+                        const V2<T>* nodeT, B4<T>* Dinv, B4<T>* Lz, B4<T>* Uz, T* vs,
+                        const int* mask, int mstride, int S, cudaStream_t st);
 // (phi, K / mu) in T for every cell of S samples
 template <class T>
 void launch_cell_inputs(const Grid& G, double mu, const double* phi, const double* K,
@@ -229,14 +240,16 @@ void launch_smooth_zline(const Grid& G, const B4<M>* J, const B4<T>* Dinv, const
 // operator, zMi and zC [S][N], and the line sweep that substitutes with
 // them (mode 1: x = 0; mode 2: r is the masked residual of x).  Lines of at
 // most kMaxLine nodes.
+// The lower and upper line blocks of node n of sample s lie at Lz[s sst + n]
+// and Uz[s sst + n].
 template <class T, class M>
-void launch_zline_factor(const Grid& G, const B4<M>* J, const B4<T>* Dinv, const uint8_t* bc,
-                         B4<T>* zMi, B4<T>* zC, const int* mask, int mstride, int S,
-                         cudaStream_t st);
+void launch_zline_factor(const Grid& G, const B4<M>* Lz, const B4<M>* Uz, size_t sst,
+                         const B4<T>* Dinv, const uint8_t* bc, B4<T>* zMi, B4<T>* zC,
+                         const int* mask, int mstride, int S, cudaStream_t st);
 // bs threads per block; spc lines of different samples per thread (1 or 2)
 template <class T, class M>
-void launch_zline_apply(const Grid& G, const B4<M>* J, const B4<T>* zMi, const B4<T>* zC,
-                        const uint8_t* bc, const V2<T>* r, const V2<T>* x, V2<T>* xo,
+void launch_zline_apply(const Grid& G, const B4<M>* Lz, size_t sst, const B4<T>* zMi,
+                        const B4<T>* zC, const uint8_t* bc, const V2<T>* r, const V2<T>* x, V2<T>* xo,
                         double omega, const int* mask, int mstride, int S, cudaStream_t st,
                         int mode, int bs = 128, int spc = 1);
 
@@ -266,6 +279,18 @@ void launch_ilu_apply(const Grid& G, const B4<M>* F, const B4<T>* Fd, const uint
                       const V2<T>* r, V2<T>* t, const V2<T>* x, V2<T>* xo, double omega,
                       int trans, int mode, const int* mask, int mstride, int S, cudaStream_t st,
                       int bs = kBS);
+
+// ---- matfree.cu ------------------------------------------------------------
+// Products with the Jacobian of launch_jacobian<float> from its inputs (nodeT,
+// cellT) instead of its stored rows.  mode 0: y = A x; 1: also partial[0] =
+// (a, y); 2: partial[0] = (y, a), partial[1] = (y, y); 3: y = a - A x.
+// Dirichlet components of y are 0.  partial [S][2][mf_blocks(G, S)]; vs:
+// device scalar |scv| / dt (launch_line_blocks).
+void launch_mf_apply(const Grid& G, const Phys& ph, const uint8_t* bc, const V2<float>* cellT,
+                     const V2<float>* nodeT, const V2<float>* x, V2<float>* y, int mode,
+                     const V2<float>* a, double* partial, const float* vs, const int* mask,
+                     int mstride, int S, cudaStream_t st);
+int mf_blocks(const Grid& G, int S);
 
 // Keeps the iterate of smallest residual: copies x into xbest for the
 // samples whose last iteration improved it (keep == 1), or x <- xbest for

@@ -447,8 +447,8 @@ void launch_smooth_zline(const Grid& G, const B4<M>* J, const B4<T>* Dinv, const
 // leave the per-sweep work.
 template <class T, class M>
 __global__ void __launch_bounds__(kBS)
-    k_zline_factor(Grid G, const B4<M>* __restrict__ J, const B4<T>* __restrict__ Dinv,
-                   const uint8_t* __restrict__ bc, B4<T>* __restrict__ zMi,
+    k_zline_factor(Grid G, const B4<M>* __restrict__ Lz, const B4<M>* __restrict__ Uz,
+                   size_t sst, const B4<T>* __restrict__ Dinv, const uint8_t* __restrict__ bc, B4<T>* __restrict__ zMi,
                    B4<T>* __restrict__ zC, const int* mask, int mstride)
 {
     const int s = blockIdx.y;
@@ -457,9 +457,8 @@ __global__ void __launch_bounds__(kBS)
     const int col = blockIdx.x * blockDim.x + threadIdx.x;
     if (col >= sz) return;
     const size_t on_ = (size_t)s * G.N;
-    const B4<M>* Js = J + (size_t)s * 27 * G.N;
-    const B4<M>* Jl = Js + (size_t)slot27(0, 0, -1) * G.N;
-    const B4<M>* Ju = Js + (size_t)slot27(0, 0, 1) * G.N;
+    const B4<M>* Jl = Lz + s * sst;
+    const B4<M>* Ju = Uz + s * sst;
     B4<T> Cp{T(0), T(0), T(0), T(0)};
     uint8_t bc_prev = 0;
     for (int k = 0; k <= G.nz; ++k) {
@@ -484,13 +483,13 @@ __global__ void __launch_bounds__(kBS)
 }
 
 template <class T, class M>
-void launch_zline_factor(const Grid& G, const B4<M>* J, const B4<T>* Dinv, const uint8_t* bc,
-                         B4<T>* zMi, B4<T>* zC, const int* mask, int mstride, int S,
-                         cudaStream_t st)
+void launch_zline_factor(const Grid& G, const B4<M>* Lz, const B4<M>* Uz, size_t sst,
+                         const B4<T>* Dinv, const uint8_t* bc, B4<T>* zMi, B4<T>* zC,
+                         const int* mask, int mstride, int S, cudaStream_t st)
 {
     count_launch(1);
     dim3 grid(nblocks((G.nx + 1) * (G.ny + 1)), S);
-    k_zline_factor<T, M><<<grid, kBS, 0, st>>>(G, J, Dinv, bc, zMi, zC, mask, mstride);
+    k_zline_factor<T, M><<<grid, kBS, 0, st>>>(G, Lz, Uz, sst, Dinv, bc, zMi, zC, mask, mstride);
 }
 
 // One damped z-line sweep with the factors of k_zline_factor (the
@@ -504,7 +503,7 @@ void launch_zline_factor(const Grid& G, const B4<M>* J, const B4<T>* Dinv, const
 // inactive sample's line is read as sample s0's and not written.
 template <class T, class M, int MODE, int SPC>
 __global__ void __launch_bounds__(kBS)
-    k_zline_apply(Grid G, const B4<M>* __restrict__ J, const B4<T>* __restrict__ zMi,
+    k_zline_apply(Grid G, const B4<M>* __restrict__ Lz, size_t sst, const B4<T>* __restrict__ zMi,
                   const B4<T>* __restrict__ zC, const uint8_t* __restrict__ bc,
                   const V2<T>* __restrict__ r, const V2<T>* __restrict__ x, V2<T>* xo, T omega,
                   const int* mask, int mstride, int S)
@@ -521,10 +520,12 @@ __global__ void __launch_bounds__(kBS)
     const int sz = (G.nx + 1) * (G.ny + 1);
     const int col = blockIdx.x * blockDim.x + threadIdx.x;
     if (col >= sz) return;
-    size_t on_[SPC];
+    size_t on_[SPC], ol_[SPC];
 #pragma unroll
-    for (int q = 0; q < SPC; ++q) on_[q] = (size_t)(act[q] ? s0 + q : s0) * G.N;
-    const size_t jl = (size_t)slot27(0, 0, -1) * G.N;
+    for (int q = 0; q < SPC; ++q) {
+        on_[q] = (size_t)(act[q] ? s0 + q : s0) * G.N;
+        ol_[q] = (size_t)(act[q] ? s0 + q : s0) * sst;
+    }
     V2<T> gp[SPC];
 #pragma unroll
     for (int q = 0; q < SPC; ++q) gp[q] = V2<T>{T(0), T(0)};
@@ -536,7 +537,7 @@ __global__ void __launch_bounds__(kBS)
 #pragma unroll
         for (int q = 0; q < SPC; ++q) {
             const V2<T> bv = r[on_[q] + n];
-            const B4<M> qL = J[on_[q] * 27 + jl + (k > 0 ? n : col)];
+            const B4<M> qL = Lz[ol_[q] + (k > 0 ? n : col)];
             const B4<T> Mi = zMi[on_[q] + n];
             T rp = (mk & BC_P) ? T(0) : bv.p;
             T rc = (mk & BC_C) ? T(0) : bv.c;
@@ -577,16 +578,16 @@ __global__ void __launch_bounds__(kBS)
 }
 
 template <class T, class M>
-void launch_zline_apply(const Grid& G, const B4<M>* J, const B4<T>* zMi, const B4<T>* zC,
-                        const uint8_t* bc, const V2<T>* r, const V2<T>* x, V2<T>* xo,
+void launch_zline_apply(const Grid& G, const B4<M>* Lz, size_t sst, const B4<T>* zMi,
+                        const B4<T>* zC, const uint8_t* bc, const V2<T>* r, const V2<T>* x, V2<T>* xo,
                         double omega, const int* mask, int mstride, int S, cudaStream_t st,
                         int mode, int bs, int spc)
 {
     count_launch(1);
     dim3 grid(nblocks((G.nx + 1) * (G.ny + 1), bs), (S + spc - 1) / spc);
 #define ELDER_ZLA(MO, SP)                                                                      \
-    k_zline_apply<T, M, MO, SP><<<grid, bs, 0, st>>>(G, J, zMi, zC, bc, r, x, xo, T(omega),   \
-                                                     mask, mstride, S)
+    k_zline_apply<T, M, MO, SP><<<grid, bs, 0, st>>>(G, Lz, sst, zMi, zC, bc, r, x, xo,       \
+                                                     T(omega), mask, mstride, S)
     if (mode == 1) {
         if (spc == 2) ELDER_ZLA(1, 2);
         else ELDER_ZLA(1, 1);
@@ -1640,17 +1641,24 @@ void launch_convert(const V2<Ts>* x, V2<Td>* y, size_t n, cudaStream_t st)
     template void launch_smooth_zline<T, typename MgType<T>::type>(                      \
         const Grid&, const B4<typename MgType<T>::type>*, const B4<T>*, const uint8_t*,  \
         const V2<T>*, const V2<T>*, V2<T>*, double, int, const int*, int, int,           \
-        cudaStream_t, int);                                                              \
-    template void launch_zline_factor<T, typename MgType<T>::type>(                      \
-        const Grid&, const B4<typename MgType<T>::type>*, const B4<T>*, const uint8_t*,  \
-        B4<T>*, B4<T>*, const int*, int, int, cudaStream_t);                             \
-    template void launch_zline_apply<T, typename MgType<T>::type>(                       \
-        const Grid&, const B4<typename MgType<T>::type>*, const B4<T>*, const B4<T>*,    \
-        const uint8_t*, const V2<T>*, const V2<T>*, V2<T>*, double, const int*, int, int,\
-        cudaStream_t, int, int, int);
+        cudaStream_t, int);
 ELDER_INST(double)
 ELDER_INST(float)
 #undef ELDER_INST
+// (line blocks stored with the multigrid matrix, or in FP32 beside the
+// matrix-free finest level of the mixed solver)
+#define ELDER_INST_ZLINE(T, M)                                                              \
+    template void launch_zline_factor<T, M>(const Grid&, const B4<M>*, const B4<M>*, size_t, \
+                                            const B4<T>*, const uint8_t*, B4<T>*, B4<T>*,    \
+                                            const int*, int, int, cudaStream_t);             \
+    template void launch_zline_apply<T, M>(const Grid&, const B4<M>*, size_t, const B4<T>*,  \
+                                           const B4<T>*, const uint8_t*, const V2<T>*,       \
+                                           const V2<T>*, V2<T>*, double, const int*, int,    \
+                                           int, cudaStream_t, int, int, int);
+ELDER_INST_ZLINE(double, double)
+ELDER_INST_ZLINE(float, __nv_bfloat16)
+ELDER_INST_ZLINE(float, float)
+#undef ELDER_INST_ZLINE
 template void launch_convert<double, float>(const V2<double>*, V2<float>*, size_t, cudaStream_t);
 template void launch_convert<float, double>(const V2<float>*, V2<double>*, size_t, cudaStream_t);
 template void launch_convert<double, double>(const V2<double>*, V2<double>*, size_t, cudaStream_t);
