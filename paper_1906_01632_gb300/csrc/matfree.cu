@@ -23,13 +23,20 @@
 //
 // Layout: a CTA owns a tile of (x, z) columns and marches along y.  A thread
 // holds one cell column: the four corners of the row behind it stay in
-// registers (as values and as (3,1)-weighted sums, so that each row's in-plane
-// sums are formed once), the next row's corners come from a shared-memory row
-// of float4 (p', c, x_p, x_c).  The contributions of a cell to the three
-// corners owned by other threads cross through shared memory.  Both
-// exchanges are double-buffered, so a row costs one __syncthreads.  The box
-// is flat (nz is the short direction), so a tile holds whole z columns on most
-// grids and only its x sides (and the ends of a y chunk) are computed twice.
+// registers, the next row's come from a shared-memory row of (p', x_p, c, x_c).
+// Rows, coefficients and the second operand arrive by asynchronous copies two
+// layers' arithmetic ahead: with the loads one layer ahead in registers (and
+// with 4 to 16 of them spilled) the warps waited for memory 2.4 of 7 cycles per
+// instruction.  A quantity of the state and the same one of x share the packed
+// FP32 instructions.  The contributions of a cell to the three corners owned by
+// other threads cross through shared memory, double-buffered, so a row costs
+// one __syncthreads.  The box is flat (nz is the short direction), so a tile
+// holds whole z columns on most grids and only its x sides (and the ends of a
+// y chunk) are computed twice.  256 threads of 128 registers, two CTAs per SM;
+// three or four smaller CTAs of fewer registers spill and are slower (518 to
+// 811 us).  64x64x16 x 256, the three kinds of product: 657, 684, 595 us with one
+// value per instruction and register prefetch, 441, 477, 414 us now, 62 % of the
+// issue slots, the FMA pipe throttling.
 #include <algorithm>
 
 #include "kernels.h"
@@ -38,7 +45,7 @@ namespace elder {
 
 namespace {
 
-constexpr int kMfThreads = 512;   // largest CTA
+constexpr int kMfThreads = 256;   // largest CTA
 constexpr int kMfResident = 512;  // threads an SM holds (128 registers each)
 
 // Tiling of a launch: ntx x ntz tiles of ox x oz output columns, nch chunks of
@@ -58,71 +65,92 @@ struct MfConst {
     float rho0, drho, drho2;
 };
 
-// (3,1) sums of a pair: (a, b) -> (3 a + b, a + 3 b)
-__device__ __forceinline__ void pass31(float& a, float& b)
+// Asynchronous copy of one word to shared memory (0 where `on` is false).
+__device__ __forceinline__ void copy_word(float* dst, const float* src, bool on)
 {
-    const float t = a + b;
-    a = fmaf(2.0f, a, t);
-    b = fmaf(2.0f, b, t);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(
+                     static_cast<unsigned>(__cvta_generic_to_shared(dst))),
+                 "l"(src), "r"(on ? 4 : 0)
+                 : "memory");
 }
 
-// The four corners (x + 2 z) of one row of a cell column and the row's
-// in-plane sums: gx[z], gz[x] the (3,1) sums of the x and z differences of p',
-// dx, dz those of x_p; C, V the (3,1) x (3,1) sums of c and x_c.
+__device__ __forceinline__ void copy_pair(V2<float>* dst, const V2<float>* src, bool on)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(
+                     static_cast<unsigned>(__cvta_generic_to_shared(dst))),
+                 "l"(src), "r"(on ? 8 : 0)
+                 : "memory");
+}
+
+__device__ __forceinline__ void copies_commit()
+{
+    asm volatile("cp.async.commit_group;" ::: "memory");
+}
+
+// All but the newest group of copies have arrived.
+__device__ __forceinline__ void copies_wait()
+{
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
+}
+
+// Two FP32 operations per instruction (the packed forms of sm_103a): a pair
+// holds a quantity of the state and the same one of x, whose sums and
+// differences are formed alike.
+__device__ __forceinline__ float2 sub2(float2 a, float2 b)
+{
+    return __ffma2_rn(b, make_float2(-1.0f, -1.0f), a);
+}
+
+// (3,1) sums of two pairs: (a, b) -> (3 a + b, a + 3 b)
+__device__ __forceinline__ void pass31(float2& a, float2& b)
+{
+    const float2 two = make_float2(2.0f, 2.0f), t = __fadd2_rn(a, b);
+    a = __ffma2_rn(two, a, t);
+    b = __ffma2_rn(two, b, t);
+}
+
+__device__ __forceinline__ void plane31(float2 (&q)[4])
+{
+    pass31(q[0], q[1]);
+    pass31(q[2], q[3]);
+    pass31(q[0], q[2]);
+    pass31(q[1], q[3]);
+}
+
+// The four corners (x + 2 z) of one row of a cell column, p = (p', x_p) and c =
+// (c, x_c), and the row's in-plane sums: gx[z], gz[x] the (3,1) sums of the x
+// and z differences of p, C the (3,1) x (3,1) sums of c.
 struct MfRow {
-    float p[4], c[4], u[4], v[4];
-    float gx[2], gz[2], dx[2], dz[2];
-    float C[4], V[4];
+    float2 p[4], c[4];
 };
 
 __device__ __forceinline__ void row_set(MfRow& r, const float4& a, const float4& b,
                                         const float4& d, const float4& e)
 {
-    r.p[0] = a.x; r.p[1] = b.x; r.p[2] = d.x; r.p[3] = e.x;
-    r.c[0] = a.y; r.c[1] = b.y; r.c[2] = d.y; r.c[3] = e.y;
-    r.u[0] = a.z; r.u[1] = b.z; r.u[2] = d.z; r.u[3] = e.z;
-    r.v[0] = a.w; r.v[1] = b.w; r.v[2] = d.w; r.v[3] = e.w;
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-        r.gx[q] = r.p[2 * q + 1] - r.p[2 * q];
-        r.dx[q] = r.u[2 * q + 1] - r.u[2 * q];
-        r.gz[q] = r.p[q + 2] - r.p[q];
-        r.dz[q] = r.u[q + 2] - r.u[q];
-    }
-    pass31(r.gx[0], r.gx[1]);
-    pass31(r.dx[0], r.dx[1]);
-    pass31(r.gz[0], r.gz[1]);
-    pass31(r.dz[0], r.dz[1]);
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        r.C[q] = r.c[q];
-        r.V[q] = r.v[q];
-    }
-    pass31(r.C[0], r.C[1]); pass31(r.C[2], r.C[3]);
-    pass31(r.C[0], r.C[2]); pass31(r.C[1], r.C[3]);
-    pass31(r.V[0], r.V[1]); pass31(r.V[2], r.V[3]);
-    pass31(r.V[0], r.V[2]); pass31(r.V[1], r.V[3]);
+    r.p[0] = make_float2(a.x, a.y); r.c[0] = make_float2(a.z, a.w);
+    r.p[1] = make_float2(b.x, b.y); r.c[1] = make_float2(b.z, b.w);
+    r.p[2] = make_float2(d.x, d.y); r.c[2] = make_float2(d.z, d.w);
+    r.p[3] = make_float2(e.x, e.y); r.c[3] = make_float2(e.z, e.w);
 }
 
-// Derivative (dm, dF) of one quarter face from its end A to B: g, d the
-// weighted differences of p' and x_p; zA, zB and wA, wB the cell sums of c and
-// x_c at the ends; cA.. the end values; kA, dA the cell's coefficients.
+// Derivative (dm, dF) of one quarter face from its end A to B: g the weighted
+// differences of p; zA, zB the cell sums of c at the ends; cA, cB the end
+// values; kA, dA the cell's coefficients.
 template <bool VERT>
-__device__ __forceinline__ void face(const MfConst& k, float kA, float dA, float g, float d,
-                                     float zA, float zB, float wA, float wB, float cA, float cB,
-                                     float vA, float vB, float& dm, float& dF)
+__device__ __forceinline__ float2 face(const MfConst& k, float kA, float dA, float2 g, float2 zA,
+                                       float2 zB, float2 cA, float2 cB)
 {
-    const float zs = zA + zB, ws = wA + wB;
-    const float rho = fmaf(k.drho128, zs, k.rho0);
-    const float drho = k.drho128 * ws;
-    const float t = kA * (VERT ? fmaf(k.gz, zs, g) : g);
-    const float s = kA * (VERT ? fmaf(k.gz, ws, d) : d);
-    const float m = rho * t;
-    dm = fmaf(rho, s, drho * t);
+    const float2 z = __fadd2_rn(zA, zB), dz = sub2(zB, zA);
+    // (rho, its derivative) and (-(K/mu) A G, its derivative)
+    const float2 rho = __ffma2_rn(make_float2(k.drho128, k.drho128), z, make_float2(k.rho0, 0.f));
+    if (VERT) g = __ffma2_rn(make_float2(k.gz, k.gz), z, g);
+    const float2 t = __fmul2_rn(make_float2(kA, kA), g);
+    const float m = rho.x * t.x;
+    const float dm = fmaf(rho.x, t.y, rho.y * t.x);
     const bool up = m >= 0.0f;
-    const float cu = up ? cA : cB, vu = up ? vA : vB;
-    const float w = fmaf(drho, zB - zA, rho * (wB - wA));
-    dF = fmaf(cu, dm, fmaf(vu, m, dA * w));
+    const float cu = up ? cA.x : cB.x, vu = up ? cA.y : cB.y;
+    const float w = fmaf(rho.y, dz.x, rho.x * dz.y);
+    return make_float2(dm, fmaf(cu, dm, fmaf(vu, m, dA * w)));
 }
 
 // One cell between the rows lo (y = j) and hi (y = j + 1): adds the face
@@ -130,72 +158,60 @@ __device__ __forceinline__ void face(const MfConst& k, float kA, float dA, float
 __device__ __forceinline__ void cell_apply(const MfConst& k, float phi, float km, const MfRow& lo,
                                            const MfRow& hi, float2 (&al)[4], float2 (&ah)[4])
 {
-    // cell sums of c and x_c: the (3,1) pass along y
-    float Zl[4], Zh[4], Wl[4], Wh[4];
+    // y faces: one per (x, z) corner, from row lo to row hi
+    float2 g[4], Zl[4], Zh[4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-        Zl[q] = lo.C[q]; Zh[q] = hi.C[q];
+        g[q] = sub2(hi.p[q], lo.p[q]);
+        // cell sums of c: the (3,1) pass along y
+        Zl[q] = lo.c[q];
+        Zh[q] = hi.c[q];
         pass31(Zl[q], Zh[q]);
-        Wl[q] = lo.V[q]; Wh[q] = hi.V[q];
-        pass31(Wl[q], Wh[q]);
     }
-    // y faces: one per (x, z) corner, from row lo to row hi
-    {
-        float g[4], d[4];
+    plane31(g);
+    plane31(Zl); plane31(Zh);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            g[q] = hi.p[q] - lo.p[q];
-            d[q] = hi.u[q] - lo.u[q];
-        }
-        pass31(g[0], g[1]); pass31(g[2], g[3]); pass31(g[0], g[2]); pass31(g[1], g[3]);
-        pass31(d[0], d[1]); pass31(d[2], d[3]); pass31(d[0], d[2]); pass31(d[1], d[3]);
-        const float kA = km * k.kA[1], dA = phi * k.dA[1];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            float dm, dF;
-            face<false>(k, kA, dA, g[q], d[q], Zl[q], Zh[q], Wl[q], Wh[q], lo.c[q], hi.c[q],
-                        lo.v[q], hi.v[q], dm, dF);
-            al[q].x += dm;
-            al[q].y += dF;
-            ah[q].x = -dm;
-            ah[q].y = -dF;
-        }
+    for (int q = 0; q < 4; ++q) {
+        const float2 f = face<false>(k, km * k.kA[1], phi * k.dA[1], g[q], Zl[q], Zh[q], lo.c[q],
+                                     hi.c[q]);
+        al[q] = __fadd2_rn(al[q], f);
+        ah[q] = make_float2(-f.x, -f.y);
     }
+    float2 gx[4], gz[4];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        gx[q] = sub2(lo.p[2 * q + 1], lo.p[2 * q]);
+        gz[q] = sub2(lo.p[q + 2], lo.p[q]);
+        gx[q + 2] = sub2(hi.p[2 * q + 1], hi.p[2 * q]);
+        gz[q + 2] = sub2(hi.p[q + 2], hi.p[q]);
+    }
+    plane31(gx);
+    plane31(gz);
     // x faces (edge at (y, z)): corners 2 z and 2 z + 1 of a row
-    {
-        const float kA = km * k.kA[0], dA = phi * k.dA[0];
 #pragma unroll
-        for (int z = 0; z < 2; ++z) {
-            float gl = lo.gx[z], gh = hi.gx[z], dl = lo.dx[z], dh = hi.dx[z];
-            pass31(gl, gh);
-            pass31(dl, dh);
-            const int A = 2 * z, B = 2 * z + 1;
-            float dm, dF;
-            face<false>(k, kA, dA, gl, dl, Zl[A], Zl[B], Wl[A], Wl[B], lo.c[A], lo.c[B], lo.v[A],
-                        lo.v[B], dm, dF);
-            al[A].x += dm; al[A].y += dF; al[B].x -= dm; al[B].y -= dF;
-            face<false>(k, kA, dA, gh, dh, Zh[A], Zh[B], Wh[A], Wh[B], hi.c[A], hi.c[B], hi.v[A],
-                        hi.v[B], dm, dF);
-            ah[A].x += dm; ah[A].y += dF; ah[B].x -= dm; ah[B].y -= dF;
-        }
+    for (int z = 0; z < 2; ++z) {
+        const float kA = km * k.kA[0], dA = phi * k.dA[0];
+        float2 gl = gx[z], gh = gx[z + 2];
+        const int A = 2 * z, B = 2 * z + 1;
+        const float2 f = face<false>(k, kA, dA, gl, Zl[A], Zl[B], lo.c[A], lo.c[B]);
+        al[A] = __fadd2_rn(al[A], f);
+        al[B] = sub2(al[B], f);
+        const float2 h = face<false>(k, kA, dA, gh, Zh[A], Zh[B], hi.c[A], hi.c[B]);
+        ah[A] = __fadd2_rn(ah[A], h);
+        ah[B] = sub2(ah[B], h);
     }
     // z faces (edge at (x, y)): corners x and x + 2 of a row
-    {
-        const float kA = km * k.kA[2], dA = phi * k.dA[2];
 #pragma unroll
-        for (int x = 0; x < 2; ++x) {
-            float gl = lo.gz[x], gh = hi.gz[x], dl = lo.dz[x], dh = hi.dz[x];
-            pass31(gl, gh);
-            pass31(dl, dh);
-            const int A = x, B = x + 2;
-            float dm, dF;
-            face<true>(k, kA, dA, gl, dl, Zl[A], Zl[B], Wl[A], Wl[B], lo.c[A], lo.c[B], lo.v[A],
-                       lo.v[B], dm, dF);
-            al[A].x += dm; al[A].y += dF; al[B].x -= dm; al[B].y -= dF;
-            face<true>(k, kA, dA, gh, dh, Zh[A], Zh[B], Wh[A], Wh[B], hi.c[A], hi.c[B], hi.v[A],
-                       hi.v[B], dm, dF);
-            ah[A].x += dm; ah[A].y += dF; ah[B].x -= dm; ah[B].y -= dF;
-        }
+    for (int x = 0; x < 2; ++x) {
+        const float kA = km * k.kA[2], dA = phi * k.dA[2];
+        float2 gl = gz[x], gh = gz[x + 2];
+        const int A = x, B = x + 2;
+        const float2 f = face<true>(k, kA, dA, gl, Zl[A], Zl[B], lo.c[A], lo.c[B]);
+        al[A] = __fadd2_rn(al[A], f);
+        al[B] = sub2(al[B], f);
+        const float2 h = face<true>(k, kA, dA, gh, Zh[A], Zh[B], hi.c[A], hi.c[B]);
+        ah[A] = __fadd2_rn(ah[A], h);
+        ah[B] = sub2(ah[B], h);
     }
 }
 
@@ -203,16 +219,20 @@ __device__ __forceinline__ void cell_apply(const MfConst& k, float phi, float km
 // partial[1] = (y, y) (partial [S][2][gridDim.x]); 3: y = a - A x.  Dirichlet
 // components of y are 0.
 template <int MODE>
-__global__ void __launch_bounds__(kMfThreads)
+__global__ void __launch_bounds__(kMfThreads, kMfResident / kMfThreads)
     k_mf_apply(Grid G, MfConst k, MfTiling t, const uint8_t* __restrict__ bc,
                const V2<float>* __restrict__ cellT, const V2<float>* __restrict__ nodeT,
                const V2<float>* __restrict__ x, V2<float>* __restrict__ y,
                const V2<float>* __restrict__ a, double* __restrict__ partial,
                const float* __restrict__ vs, const int* mask, int mstride)
 {
-    __shared__ float4 nd[2][kMfThreads];
-    __shared__ float2 ct[2][3][kMfThreads];
-    __shared__ float ph[2][kMfThreads];
+    // the next row's (p', x_p, c, x_c); what a thread's cells add to the
+    // corners of others: (1, 0) and (0, 1) in ca, (1, 1) in cb, the cells' phi in
+    // cp; entry kMfThreads stays zero (a side without cells)
+    __shared__ float4 nd[4][kMfThreads], ca[2][kMfThreads + 1];
+    __shared__ float2 cb[2][kMfThreads + 1];
+    __shared__ float cp[2][kMfThreads + 1];
+    __shared__ V2<float> cl[4][kMfThreads], sa[4][kMfThreads];
     __shared__ double red[32];
     const int s = blockIdx.y;
     if (mask != nullptr && mask[(size_t)s * mstride] == 0) return;
@@ -233,101 +253,101 @@ __global__ void __launch_bounds__(kMfThreads)
     const int gx = xs + tx, gz = zs + tz;
     const bool cell = in && tx < wx - 1 && tz < wz - 1;
     const bool out = in && gx >= x0 && gx < x1 && gz >= z0 && gz < z1;
-    const bool hasx = tx > 0, hasz = tz > 0;
-    const size_t on = (size_t)s * G.N;
-    const int n0 = in ? gx + pl * gz : 0;             // node of row 0
-    const int e0 = cell ? gx + G.nx * G.ny * gz : 0;  // cell of row 0
-    const V2<float>* ns = nodeT + on + n0;
-    const V2<float>* xv = x + on + n0;
-    const V2<float>* cs = cellT + (size_t)s * G.C + e0;
+    // node and cell of row 0 (32-bit offsets: registers decide the occupancy
+    // here; a batch of 2^32 nodes would not fit the device)
+    const unsigned n0 = (unsigned)s * (unsigned)G.N + (in ? gx + pl * gz : 0);
+    const unsigned e0 = (unsigned)s * (unsigned)G.C + (cell ? gx + G.nx * G.ny * gz : 0);
     const int js = max(j0 - 1, 0), je = min(j1 - 1, G.ny - 1);  // layers of cells
-    auto load = [&](int j) {
-        float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (in) {
-            const V2<float> st = ns[nx1 * j], w = xv[nx1 * j];
-            q = make_float4(st.p, st.c, w.p, w.c);
+    // row j of the nodes, the coefficients of layer j - 1 and a's row j - 1 into
+    // their buffers, one group per row (empty past the last); the nodes word
+    // by word, into the order of the pairs
+    auto copy_row = [&](int j) {
+        const int b = j & 3;
+        if (j <= je + 1) {
+            float* d = &nd[b][tid].x;
+            const V2<float>*st = nodeT + (n0 + nx1 * j), *w = x + (n0 + nx1 * j);
+            copy_word(d, &st->p, in);
+            copy_word(d + 1, &w->p, in);
+            copy_word(d + 2, &st->c, in);
+            copy_word(d + 3, &w->c, in);
         }
-        return q;
+        if (j > js && j <= je + 1)
+            copy_pair(&cl[b][tid], cellT + (e0 + G.nx * (j - 1)), cell);
+        if (MODE != 0 && j > js && j <= j1)
+            copy_pair(&sa[b][tid], a + (n0 + nx1 * (j - 1)), out);
+        copies_commit();
     };
+    // neighbours: the cell's corners ahead, the cells' sides behind
     const int R = tid + (cell ? 1 : 0), U = tid + (cell ? wx : 0),
               D = tid + (cell ? wx + 1 : 0);
+    const int bX = tx > 0 ? tid - 1 : kMfThreads, bZ = tz > 0 ? tid - wx : kMfThreads,
+              bD = tx > 0 && tz > 0 ? tid - wx - 1 : kMfThreads;
     double d0 = 0.0, d1 = 0.0;
-    float4 own = load(js), nxt = load(js + 1);
-    nd[js & 1][tid] = own;
-    nd[(js + 1) & 1][tid] = nxt;
-    V2<float> co{0.f, 0.f};
-    if (cell) co = cs[G.nx * js];
+    if (tid < 2) {
+        ca[tid][kMfThreads] = make_float4(0.f, 0.f, 0.f, 0.f);
+        cb[tid][kMfThreads] = make_float2(0.f, 0.f);
+        cp[tid][kMfThreads] = 0.f;
+    }
+    copy_row(js);
+    copy_row(js + 1);
+    copy_row(js + 2);
+    copies_wait();  // rows js and js + 1
     __syncthreads();
     MfRow r0, r1;
-    row_set(r0, own, nd[js & 1][R], nd[js & 1][U], nd[js & 1][D]);
-    __syncthreads();  // the first layer overwrites row js
+    row_set(r0, nd[js & 3][tid], nd[js & 3][R], nd[js & 3][U], nd[js & 3][D]);
     float2 al[4], ah[4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) al[q] = make_float2(0.f, 0.f);
     float phl = 0.f;  // phi of the cell behind the row
+    auto share = [&](int b, float phs) {
+        ca[b][tid] = make_float4(al[1].x, al[1].y, al[2].x, al[2].y);
+        cb[b][tid] = al[3];
+        cp[b][tid] = phs;
+    };
     // row j's sums gathered from the cells around it and written
-    auto emit = [&](int j, const float2& mine, float cn, float vn) {
+    auto emit = [&](int j, float phs, float2 c, int mk) {
         const int b = j & 1;
-        float yp = mine.x, yc = mine.y, phs = ph[b][tid];
-        if (hasx) {
-            const float2 w = ct[b][0][tid - 1];
-            yp += w.x; yc += w.y;
-            phs += ph[b][tid - 1];
-        }
-        if (hasz) {
-            const float2 w = ct[b][1][tid - wx];
-            yp += w.x; yc += w.y;
-            phs += ph[b][tid - wx];
-        }
-        if (hasx && hasz) {
-            const float2 w = ct[b][2][tid - wx - 1];
-            yp += w.x; yc += w.y;
-            phs += ph[b][tid - wx - 1];
-        }
+        const float2 w0 = *reinterpret_cast<const float2*>(&ca[b][bX].x);
+        const float2 w1 = *reinterpret_cast<const float2*>(&ca[b][bZ].z);
+        const float2 w2 = cb[b][bD];
+        float yp = (al[0].x + w0.x) + (w1.x + w2.x), yc = (al[0].y + w0.y) + (w1.y + w2.y);
+        phs = (phs + cp[b][bX]) + (cp[b][bZ] + cp[b][bD]);
         if (!out) return;
-        const int n = n0 + nx1 * j;
-        const float vd = phs * vscale * vn;
-        yp = fmaf(vd, k.drho, yp);
-        yc = fmaf(vd, fmaf(k.drho2, cn, k.rho0), yc);
+        const float vd = phs * vscale * c.y;
         V2<float> av{0.f, 0.f};
-        if (MODE != 0) av = a[on + n];
+        if (MODE != 0) av = sa[(j + 1) & 3][tid];
+        yp = fmaf(vd, k.drho, yp);
+        yc = fmaf(vd, fmaf(k.drho2, c.x, k.rho0), yc);
         if (MODE == 3) { yp = av.p - yp; yc = av.c - yc; }
-        const uint8_t m = bc[n];
-        if (m & BC_P) yp = 0.f;
-        if (m & BC_C) yc = 0.f;
-        y[on + n] = V2<float>{yp, yc};
+        if (mk & BC_P) yp = 0.f;
+        if (mk & BC_C) yc = 0.f;
+        y[n0 + nx1 * j] = V2<float>{yp, yc};
         if (MODE == 1 || MODE == 2) d0 += dot2(av.p, av.c, yp, yc);
         if (MODE == 2) d1 += dot2(yp, yc, yp, yc);
     };
     // one layer: cells between row j (state lo) and row j + 1 (state hi)
+    int mk = 0;  // the Dirichlet bits of row j
     auto layer = [&](int j, MfRow& lo, MfRow& hi) {
-        // the row after next and the next layer's coefficients, used after
-        // this layer's arithmetic
-        float4 nn = nxt;
-        V2<float> cn{0.f, 0.f};
-        if (j < je) {
-            nn = load(j + 2);
-            if (cell) cn = cs[G.nx * (j + 1)];
-        }
-        const int b = j & 1, h = (j + 1) & 1;
-        row_set(hi, nxt, nd[h][R], nd[h][U], nd[h][D]);
+        // three rows ahead of the one behind: two layers' arithmetic hide the
+        // copies (over row j - 1, whose last reader was the previous layer)
+        copy_row(j + 3);
+        if (out) mk = bc[gx + pl * gz + nx1 * j];
+        const int b = j & 1, h = (j + 1) & 3;
+        row_set(hi, nd[h][tid], nd[h][R], nd[h][U], nd[h][D]);
+        const V2<float> co = cl[h][tid];
         cell_apply(k, co.p, co.c, lo, hi, al, ah);
         if (!cell) {
 #pragma unroll
             for (int q = 0; q < 4; ++q) ah[q] = al[q] = make_float2(0.f, 0.f);
         }
-        ct[b][0][tid] = al[1];
-        ct[b][1][tid] = al[2];
-        ct[b][2][tid] = al[3];
-        ph[b][tid] = phl + co.p;
-        nd[b][tid] = nn;  // row j was read as the previous layer's far row
+        const float phs = phl + co.p;
+        share(b, phs);
+        copies_wait();
         __syncthreads();
-        if (j >= j0) emit(j, al[0], lo.c[0], lo.v[0]);
+        if (j >= j0) emit(j, phs, lo.c[0], mk);
 #pragma unroll
         for (int q = 0; q < 4; ++q) al[q] = ah[q];
         phl = co.p;
-        co = cn;
-        nxt = nn;
     };
     int j = js;
     for (; j + 1 <= je; j += 2) {
@@ -337,16 +357,13 @@ __global__ void __launch_bounds__(kMfThreads)
     if (j <= je) {
         layer(j, r0, r1);
         r0.c[0] = r1.c[0];
-        r0.v[0] = r1.v[0];
     }
     if (j1 == G.ny + 1) {  // the last row of nodes has cells behind it only
-        const int b = G.ny & 1;
-        ct[b][0][tid] = al[1];
-        ct[b][1][tid] = al[2];
-        ct[b][2][tid] = al[3];
-        ph[b][tid] = phl;
+        if (out) mk = bc[gx + pl * gz + nx1 * G.ny];
+        share(G.ny & 1, phl);
+        asm volatile("cp.async.wait_all;" ::: "memory");
         __syncthreads();
-        emit(G.ny, al[0], r0.c[0], r0.v[0]);
+        emit(G.ny, phl, r0.c[0], mk);
     }
     if (MODE == 1 || MODE == 2) {
         const double s0 = block_sum(d0, red);
