@@ -1489,25 +1489,89 @@ void launch_newton_restore_failed(const Grid& G, double* p, double* c,
 // for stability: with d_i = c_i - c_0, S1 = sum w d, S2 = sum w d^2,
 // W = sum w: mean = c_0 W + S1 and sum w (mean - c)^2 =
 // (mean - c_0)^2 W - 2 (mean - c_0) S1 + S2.
+//
+// Bound by FP64 issue (1/64 of the FP32 rate here): 7 operations per value
+// (difference, weighted difference, both sums, W, the threshold comparison
+// and its sum) took 264 us for 256 fields of 71,825 nodes, 22 us of them
+// memory time.  Now 3 for equal weights (the weight is applied to the sums; 158
+// us) and 4 or 5 for given ones: W is formed once per block, the comparison is an
+// integer one, the equal-weight count an integer.  kMomSplit threads of
+// different warps share a node, each over every kMomSplit-th field, to keep
+// the FP64 pipe fed; their sums meet in shared memory in a fixed order.
+constexpr int kMomSplit = 4;
+constexpr int kMomNodes = kBS / kMomSplit;  // nodes per block
+
+// x > t for finite or infinite x, t of either sign, false for NaN (integer
+// operations: bit patterns as two's-complement numbers order like the values)
+__device__ __forceinline__ long long order_key(double x)
+{
+    const long long b = __double_as_longlong(x);
+    return b < 0 ? (long long)(0x8000000000000000ull - (unsigned long long)b) : b;
+}
+
+__device__ __forceinline__ bool exceeds(double x, long long tkey)
+{
+    constexpr long long inf = 0x7FF0000000000000ll;
+    const long long k = order_key(x);
+    return k > tkey && k <= inf;
+}
+
+template <bool WEIGHTED>
 __global__ void __launch_bounds__(kBS)
-    k_moments(int N, int S, const double* __restrict__ c,
+    k_moments(int N, int S, double inv, const double* __restrict__ c,
               const double* __restrict__ w, double threshold,
               double* __restrict__ mean, double* __restrict__ var,
               double* __restrict__ pexc)
 {
-    const int n = blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= N) return;
-    const double c0 = c[n];
-    const double wu = 1.0 / S;
-    double S1 = 0.0, S2 = 0.0, W = 0.0, P = 0.0;
-    for (int s = 0; s < S; ++s) {
-        const double ws = w ? __ldg(w + s) : wu;
-        const double cv = __ldcs(c + (size_t)s * N + n);
-        const double d = cv - c0;
-        S1 = fma(ws, d, S1);
-        S2 = fma(ws * d, d, S2);
-        W += ws;
-        if (cv > threshold) P += ws;
+    __shared__ double red[32];
+    __shared__ double part[3][kMomSplit][kMomNodes];
+    const int q = threadIdx.x / kMomNodes, l = threadIdx.x % kMomNodes;
+    const int n = blockIdx.x * kMomNodes + l;
+    double W = 1.0;
+    if (WEIGHTED) {
+        W = 0.0;
+        for (int s = threadIdx.x; s < S; s += kBS) W += w[s];
+        W = block_sum(W, red);
+    }
+    // (a NaN threshold is exceeded by nothing)
+    const long long tkey = threshold == threshold ? order_key(threshold) : 0x7FFFFFFFFFFFFFFFll;
+    double S1 = 0.0, S2 = 0.0, P = 0.0, c0 = 0.0;
+    if (n < N) {
+        c0 = c[n];
+        int count = 0;
+        const double* cn = c + n;
+#pragma unroll 8
+        for (int s = q; s < S; s += kMomSplit) {
+            const double cv = __ldcs(cn + (size_t)s * N);
+            const double d = cv - c0;
+            if (WEIGHTED) {
+                const double ws = __ldg(w + s), wd = ws * d;
+                S1 += wd;
+                S2 = fma(wd, d, S2);
+                if (exceeds(cv, tkey)) P += ws;
+            } else {
+                S1 += d;
+                S2 = fma(d, d, S2);
+                count += exceeds(cv, tkey) ? 1 : 0;
+            }
+        }
+        if (!WEIGHTED) P = (double)count;
+    }
+    part[0][q][l] = S1;
+    part[1][q][l] = S2;
+    part[2][q][l] = P;
+    __syncthreads();
+    if (q != 0 || n >= N) return;
+#pragma unroll
+    for (int r = 1; r < kMomSplit; ++r) {
+        S1 += part[0][r][l];
+        S2 += part[1][r][l];
+        P += part[2][r][l];
+    }
+    if (!WEIGHTED) {  // (inv: 1 / S; all of S fields count exactly 1)
+        S1 *= inv;
+        S2 *= inv;
+        P = P == (double)S ? 1.0 : P * inv;
     }
     const double m = fma(c0, W, S1);
     const double dm = m - c0;
@@ -1521,7 +1585,11 @@ void launch_moments(int N, int S, const double* c, const double* w,
                     double* pexc, cudaStream_t st)
 {
     count_launch(1);
-    k_moments<<<nblocks(N), kBS, 0, st>>>(N, S, c, w, threshold, mean, var, pexc);
+    const int grid = nblocks(N, kMomNodes);
+    if (w)
+        k_moments<true><<<grid, kBS, 0, st>>>(N, S, 1.0 / S, c, w, threshold, mean, var, pexc);
+    else
+        k_moments<false><<<grid, kBS, 0, st>>>(N, S, 1.0 / S, c, w, threshold, mean, var, pexc);
 }
 
 // ---------------------------------------------------------------------------
