@@ -28,6 +28,7 @@ namespace {
 constexpr int kGpcMaxM = 8;      // stochastic dimensions
 constexpr int kGpcMaxDeg = 16;   // largest degree in one variable
 constexpr int kGpcBS = 128;      // threads per block
+constexpr int kGpcProjMax = 256; // threads per block of the projection
 constexpr int kGpcChunk = 128;   // samples per shared-memory chunk (even)
 
 // P_0..P_n at x by (k+1) P_{k+1} = (2k+1) x P_k - k P_{k-1} (Appendix A).
@@ -36,6 +37,19 @@ __host__ __device__ inline void legendre_all(int n, double x, double* P)
     P[0] = 1.0;
     if (n >= 1) P[1] = x;
     for (int k = 1; k < n; ++k) P[k + 1] = ((2 * k + 1) * x * P[k] - k * P[k - 1]) / (k + 1);
+}
+
+// The same with the recurrence's ratios as constants (no division).
+__device__ inline void legendre_ratios(int n, double x, double* P)
+{
+    P[0] = 1.0;
+    if (n >= 1) P[1] = x;
+#pragma unroll
+    for (int k = 1; k < kGpcMaxDeg; ++k) {
+        if (k < n)
+            P[k + 1] = fma((double(2 * k + 1) / double(k + 1)) * x, P[k],
+                           -(double(k) / double(k + 1)) * P[k - 1]);
+    }
 }
 
 // FP32 recurrence for the surrogate evaluation (its sums are FP32 anyway;
@@ -49,51 +63,83 @@ __device__ inline void legendre_all_f(int n, float x, float* P)
 
 // coef[t][n] = sum_i Bq[t][i] u[i][n] with Bq = 0.5^M w_i P_t(theta_i) / Q_t
 // (eq. PCEcoef); TP >= T accumulators per thread.
-template <int TP>
-__global__ void __launch_bounds__(kGpcBS)
+//
+// Bound by FP64 issue: T fused multiply-adds per point and node (0.51 ms for
+// 125 x 71,825 x 35).  The table is formed once per CTA, a point per thread (its
+// Legendre values once, 1 / Q_t = prod (2 beta_j + 1) as a product, no
+// division per entry), and a CTA's warps take groups of 32 nodes in turn, so
+// that the grid is a few CTAs per SM instead of one per 128 nodes.  With a
+// table per 128 nodes, its entries formed one by one with four divisions each,
+// the call took 1068 us, now 740 us.
+//
+// PAIR: rows of an even number LD of entries, two per shared-memory load.
+template <int TP, bool PAIR>
+__global__ void __launch_bounds__(kGpcProjMax)
     k_gpc_project(int M, int T, const int32_t* __restrict__ beta, int Nq,
                   const double* __restrict__ theta, const double* __restrict__ w, int N,
                   const double* __restrict__ u, double* __restrict__ coef,
                   double* __restrict__ mean, double* __restrict__ var, int maxdeg)
 {
-    extern __shared__ double sh[];
-    double* Bq = sh;               // [T][Nq]
-    double* Qt = sh + T * Nq;      // [T]
-    for (int q = threadIdx.x; q < T * Nq; q += blockDim.x) {
-        const int t = q / Nq, i = q % Nq;
-        double P1[kGpcMaxM * (kGpcMaxDeg + 1)];
-        double v = 1.0, Q = 1.0;
-        for (int j = 0; j < M; ++j) {
-            const int b = min(max((int)beta[t * M + j], 0), maxdeg);
-            legendre_all(b, theta[(size_t)i * M + j], P1 + j * (kGpcMaxDeg + 1));
-            v *= P1[j * (kGpcMaxDeg + 1) + b];
-            Q *= 1.0 / (2.0 * b + 1.0);
-        }
-        Bq[q] = ldexp(w[i] * v / Q, -M);
-        if (i == 0) Qt[t] = Q;
+    extern __shared__ __align__(16) double sh[];
+    const int LD = PAIR ? T + (T & 1) : T;
+    double* Bq = sh;               // [Nq][LD]
+    double* Rt = sh + (size_t)Nq * LD;  // [T] 1 / Q_t = prod (2 beta_j + 1)
+    double* Qt = Rt + T;                // [T]
+    for (int t = threadIdx.x; t < T; t += blockDim.x) {
+        double r = 1.0;
+        for (int j = 0; j < M; ++j)
+            r *= 2 * min(max((int)beta[t * M + j], 0), maxdeg) + 1;
+        Rt[t] = r;
+        Qt[t] = 1.0 / r;
     }
     __syncthreads();
-    const int n = blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= N) return;
-    double acc[TP];
-#pragma unroll
-    for (int t = 0; t < TP; ++t) acc[t] = 0.0;
-    for (int i = 0; i < Nq; ++i) {
-        const double ui = u[(size_t)i * N + n];
-#pragma unroll
-        for (int t = 0; t < TP; ++t)
-            if (t < T) acc[t] = fma(Bq[t * Nq + i], ui, acc[t]);
-    }
-    double vs = 0.0;
-#pragma unroll
-    for (int t = 0; t < TP; ++t) {
-        if (t < T) {
-            coef[(size_t)t * N + n] = acc[t];
-            if (t > 0) vs += Qt[t] * acc[t] * acc[t];
+    for (int i = threadIdx.x; i < Nq; i += blockDim.x) {
+        double P1[kGpcMaxM * (kGpcMaxDeg + 1)];
+        for (int j = 0; j < M; ++j)
+            legendre_ratios(maxdeg, theta[(size_t)i * M + j], P1 + j * (kGpcMaxDeg + 1));
+        const double wi = ldexp(w[i], -M);
+        for (int t = 0; t < T; ++t) {
+            double v = wi;
+            for (int j = 0; j < M; ++j)
+                v *= P1[j * (kGpcMaxDeg + 1) + min(max((int)beta[t * M + j], 0), maxdeg)];
+            Bq[(size_t)i * LD + t] = v * Rt[t];
         }
+        for (int t = T; t < LD; ++t) Bq[(size_t)i * LD + t] = 0.0;
     }
-    if (mean) mean[n] = acc[0];
-    if (var) var[n] = vs;
+    __syncthreads();
+    const int lane = threadIdx.x & 31;
+    const int warps = blockDim.x >> 5;
+    for (int g = blockIdx.x * warps + (threadIdx.x >> 5); g * 32 < N; g += gridDim.x * warps) {
+        const int n = g * 32 + lane;
+        if (n >= N) break;
+        double acc[TP];
+#pragma unroll
+        for (int t = 0; t < TP; ++t) acc[t] = 0.0;
+        for (int i = 0; i < Nq; ++i) {
+            const double ui = __ldcs(u + (size_t)i * N + n);
+#pragma unroll
+            for (int t = 0; t < TP; t += 2) {
+                if (!PAIR) {
+                    if (t < T) acc[t] = fma(Bq[(size_t)i * LD + t], ui, acc[t]);
+                    if (t + 1 < T) acc[t + 1] = fma(Bq[(size_t)i * LD + t + 1], ui, acc[t + 1]);
+                } else if (t < T) {
+                    const double2 b = *reinterpret_cast<const double2*>(Bq + (size_t)i * LD + t);
+                    acc[t] = fma(b.x, ui, acc[t]);
+                    acc[t + 1] = fma(b.y, ui, acc[t + 1]);
+                }
+            }
+        }
+        double vs = 0.0;
+#pragma unroll
+        for (int t = 0; t < TP; ++t) {
+            if (t < T) {
+                coef[(size_t)t * N + n] = acc[t];
+                if (t > 0) vs = fma(acc[t] * acc[t], Qt[t], vs);
+            }
+        }
+        if (mean) mean[n] = acc[0];
+        if (var) var[n] = vs;
+    }
 }
 
 // Surrogate at Ns points for the listed nodes; counts of values above the
@@ -837,22 +883,52 @@ int elder_gpc_project(int M, int T, const int32_t* beta, int maxdeg, int Nq, con
         set_static_error("elder_gpc_project: bad argument");
         return ELDER_EINVAL;
     }
-    const size_t smem = sizeof(double) * ((size_t)T * Nq + T);
-    if (smem > 200 * 1024) {
+    if (sizeof(double) * ((size_t)T * Nq + T) > 200 * 1024) {
         set_static_error("elder_gpc_project: T * Nq too large for one block's table");
         return ELDER_EINVAL;
     }
     cudaStream_t st = (cudaStream_t)stream;
-    const int grid = (N + kGpcBS - 1) / kGpcBS;
     const int TP = round_tp(T);
+    // rows of an even length where that fits the shared memory
+    auto bytes = [&](int ld) { return sizeof(double) * ((size_t)ld * Nq + 2 * T); };
+    const bool pair = bytes(T + (T & 1)) <= 224 * 1024;
+    const size_t smem = bytes(pair ? T + (T & 1) : T);
+    // CTAs of warps per SM that share the groups of 32 nodes most evenly, 8 to
+    // 16 warps (the FP64 pipe is full with 8; 16 of up to 128 registers fit, 12
+    // of the larger tables), in up to three CTAs where their tables fit.
+    int dev = 0, sms = 152;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int groups = (N + 31) / 32;
+    const int most = TP <= 40 ? 16 : 12;
+    int ctas = 1, wpc = 8;
+    long long least = -1;
+    for (int c = 1; c <= 3 && c * smem <= 200 * 1024; ++c)
+        for (int q = kGpcProjMax / 32; q >= 2; --q) {
+            if (c * q > most || c * q < 8) continue;
+            const long long per = (long long)sms * c * q;
+            const long long cost = (groups + per - 1) / per * c * q;
+            if (least < 0 || cost < least) {
+                least = cost;
+                ctas = c;
+                wpc = q;
+            }
+        }
+    const int threads = wpc * 32;
+    const int grid = std::max(1, std::min(ctas * sms, (groups + wpc - 1) / wpc));
     cudaError_t e = cudaSuccess;
+#define ELDER_GPC_PROJ2(TPV, PR)                                                                \
+    do {                                                                                        \
+        e = cudaFuncSetAttribute(k_gpc_project<TPV, PR>,                                        \
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);       \
+        if (e == cudaSuccess)                                                                   \
+            k_gpc_project<TPV, PR><<<grid, threads, smem, st>>>(M, T, beta, Nq, theta, w, N, u, \
+                                                                coef, mean, var, maxdeg);       \
+    } while (0)
 #define ELDER_GPC_PROJ(TPV)                                                                     \
     do {                                                                                        \
-        e = cudaFuncSetAttribute(k_gpc_project<TPV>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
-                                 (int)smem);                                                   \
-        if (e == cudaSuccess)                                                                   \
-            k_gpc_project<TPV><<<grid, kGpcBS, smem, st>>>(M, T, beta, Nq, theta, w, N, u, coef, \
-                                                           mean, var, maxdeg);                  \
+        if (pair) ELDER_GPC_PROJ2(TPV, true);                                                   \
+        else ELDER_GPC_PROJ2(TPV, false);                                                       \
     } while (0)
     switch (TP) {
         case 8: ELDER_GPC_PROJ(8); break;
@@ -865,6 +941,7 @@ int elder_gpc_project(int M, int T, const int32_t* beta, int maxdeg, int Nq, con
         default: ELDER_GPC_PROJ(64); break;
     }
 #undef ELDER_GPC_PROJ
+#undef ELDER_GPC_PROJ2
     count_launch(1);
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) {

@@ -196,3 +196,27 @@ def test_tensor_engine_many_tiles_and_slices(E):
     hi = (vals > 0.5 - delta).sum(0)
     got = np.rint(tc[pick] * Ns)
     assert ((got >= lo) & (got <= hi)).all()
+
+
+# terms 1, 2 (even rows), 35 (odd, padded), 56; points fewer and more than a
+# block's threads; 5 terms at 5,000 points (rows not padded: they would not fit);
+# nodes short of a warp, of a group of CTAs, and many groups per warp
+@pytest.mark.parametrize("M,p,Nq,N", [(1, 0, 3, 5), (1, 1, 700, 31), (3, 4, 125, 40000),
+                                      (3, 5, 216, 161), (1, 4, 5000, 70), (3, 4, 729, 33)])
+def test_projection_tables_and_groups(E, M, p, Nq, N):
+    beta = G.multi_indices(M, p)
+    rng = np.random.default_rng(Nq + N)
+    th = rng.uniform(-1, 1, (Nq, M))
+    w = rng.uniform(0, 2.0**M / Nq, Nq)
+    u = rng.uniform(0, 1, (Nq, N))
+    coef, mean, var = E.elder_gpc_project(Ti(beta), Td(th), Td(w), Td(u))
+    c_ref = G.project(u, th, w, beta)
+    m_ref, v_ref = G.mean_var(c_ref, beta)
+    # a coefficient is a sum of Nq terms of magnitude up to w (2 beta + 1)...:
+    # a few roundings per term
+    size = np.abs(G.project(np.ones((Nq, 1)), th, np.abs(w), 0 * beta[:1])).max()
+    scale = size * np.prod(2.0 * beta + 1.0, axis=1).max()
+    tol = 8 * (Nq**0.5 + 8 * p + 8) * 2.0**-53 * scale
+    assert np.abs(coef.cpu().numpy() - c_ref).max() <= tol
+    assert np.abs(mean.cpu().numpy() - m_ref).max() <= tol
+    assert np.abs(var.cpu().numpy() - v_ref).max() <= 4 * beta.shape[0] * tol * max(1.0, scale)
