@@ -114,8 +114,8 @@ typedef struct {
                                  cached for the 4 most recent argument sets
                                  (array pointers, S, dt, Newton start)      */
     int autotune;             /* 1 (default): time the candidates (threads
-                                 per block; for the multigrid residual and
-                                 the z-line sweep also 1 or 2 samples per
+                                 per block; for the multigrid residual also
+                                 1 or 2 samples per
                                  CTA) of the stencil kernels on the first
                                  step; 0: defaults (one sample per CTA);
                                  2: two samples per CTA without timing     */
@@ -358,13 +358,13 @@ int elder_profile(elder_ctx* ctx, int on);
  * counts every array the kernel must touch once (neighbour reuse of a
  * vector is free).  Per node, with T the vector entry size (8 FP64, 4
  * mixed) and Mz the multigrid matrix entry size (8 FP64, 2 mixed):
- *   SMOOTH  108 Mz + 10 T + 1    SMOOTH0  8 T + 1 (+ 8 Mz z-line)
+ *   SMOOTH  108 Mz + 10 T + 1    SMOOTH0  8 T + 1 (z-line: 16 T + 1)
  *   SPMV    108 T  + 6 T + 1     MGRES    108 Mz + 6 T + 1
  *   RESIDUAL 49 + 16 C/N         JACOBIAN 108 T + 108 Mz + 4 T + 17 + 16 C/N
  * The finest level of the mixed solver under the z-line smoother stores no
  * matrix (products from the state and the coefficients), there
- *   SMOOTH0 16 T + 1    SPMV, MGRES 8 T + 2 T C/N + 1
- *   JACOBIAN 36 T + 18 + 2 T C/N   SMOOTH 26 T + 2 T C/N + 2.
+ *   SPMV, MGRES 8 T + 2 T C/N + 1
+ *   JACOBIAN 40 T + 18 + 2 T C/N   SMOOTH 26 T + 2 T C/N + 2.
  * (the Jacobian writes the Krylov and the multigrid copies of J and the
  * inverse diagonal blocks; the residual reads p, c, c_old, phi, K and writes
  * R).  Flops: the FP64 residual counts 266 C/N + 75 of its factored face
@@ -386,7 +386,8 @@ int elder_launch_count(int64_t* launches);
  * ELDER_K_MGRES (the multigrid residual; candidates 128, 256, 512 threads)
  * and ELDER_K_SMOOTH0 (the z-line sweep from x = 0; candidates 64, 128, 256
  * threads) ms receives the measured milliseconds per launch of the 6
- * candidates [samples per CTA 1, 2][threads ascending], 0 when not tuned;
+ * candidates [samples per CTA 1, 2][threads ascending], 0 when not tuned (the
+ * sweep has one line set per CTA: the last 3 are 0);
  * for the other classes 0.  Timed on the first step of a context (3
  * launches after a warm-up, CUDA events) on its level-0 operator with all
  * samples active.  Host outputs; any may be NULL. */

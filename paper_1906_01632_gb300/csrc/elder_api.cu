@@ -154,7 +154,7 @@ template <class T> struct Solver : SolverBase {
     B4<T>* J0 = nullptr;           // level-0 Krylov operator (T)
     std::vector<B4<M>*> Jm;        // multigrid matrices per level (M)
     std::vector<B4<T>*> Dinv;      // inverse interior diagonal blocks per level
-    std::vector<B4<T>*> zMi, zC;   // block-LU factors of the vertical lines per level
+    std::vector<B4<T>*> zMi, zA, zC;  // factors of the vertical lines per level
     std::vector<B4<M>*> F;         // multicolour ILU factors per level (ILU smoother)
     std::vector<B4<T>*> Fd;        // their inverse pivot blocks
     std::vector<V2<T>*> mb, mx, mx2, mr;  // multigrid vectors per level
@@ -225,7 +225,7 @@ struct elder_ctx {
     double* cval = nullptr;            // level 0 [N]
     std::vector<double*> phi, K, pl, cl;  // levels >= 1: [S][C], [S][N]
     double *p_old = nullptr, *c_old = nullptr, *pt = nullptr, *ct = nullptr;
-    V2<double> *R = nullptr, *Rt = nullptr, *tmp2 = nullptr;
+    V2<double> *R = nullptr, *Rt = nullptr;
     double* partial = nullptr;         // [S][2][nblk0]
     double* partial2 = nullptr;
     double* partial3 = nullptr;
@@ -308,8 +308,8 @@ double model_bytes(int cls, int T, int Mz, const Grid& G, int line, bool mf)
     // (for the Jacobian class: Mz of the multigrid copy, T of the Krylov copy
     // or 0 when the level has none).  line (SMOOTH0): 1 the z-line sweep that
     // factors as it goes, reading the two vertical line blocks of J besides
-    // Dinv; 2 the sweep with the assembly's line factors (zMi, zC and the
-    // lower line block); 3 the multicolour ILU sweep from x = 0 (both
+    // Dinv; 2 the sweep with the assembly's line factors (zMi, zA, zC); 3 the
+    // multicolour ILU sweep from x = 0 (both
     // triangular solves: the 26 factor blocks, the inverse pivot, b, the
     // scratch vector written, read and written again, x_out, bc twice).
     // line (JACOBIAN): bit 0 with the line factorisation, bit 1 with the ILU
@@ -323,29 +323,29 @@ double model_bytes(int cls, int T, int Mz, const Grid& G, int line, bool mf)
     if (mf) {
         switch (cls) {
         case ELDER_K_SMOOTH: return mf_inputs + (6 + 4 + 4 + 4 + 6) * T + 2;
-        case ELDER_K_SMOOTH0: return (4 + 4 + 4 + 2 + 2) * T + 1;  // zMi, zC, L, b, xo, bc
+        case ELDER_K_SMOOTH0: return (4 + 4 + 4 + 2 + 2) * T + 1;  // zMi, zA, zC, b, xo, bc
         case ELDER_K_SPMV: return mf_inputs + (2 + 2 + 2) * T + 1;   // x, y, a, bc
         case ELDER_K_MGRES: return mf_inputs + (2 + 2 + 2) * T + 1;  // x, b, r, bc
         case ELDER_K_JACOBIAN:
             // node inputs; Dinv, L, U written; line factors: they and bc
-            // read, zMi, zC written
-            return 16 + 2 * T + mf_inputs + 1 + 12 * T + (12 + 8) * T + 1;
+            // read, zMi, zA, zC written
+            return 16 + 2 * T + mf_inputs + 1 + 12 * T + (12 + 12) * T + 1;
         }
     }
     switch (cls) {
     case ELDER_K_SMOOTH: return 108 * Mz + (4 + 2 + 2 + 2) * T + 1;  // J, Dinv, b, x, xo, bc
     case ELDER_K_SMOOTH0:
         if (line == 3) return 104 * Mz + (4 + 2 + 2 + 2 + 2 + 2) * T + 2;
-        if (line == 2) return (4 + 4 + 2 + 2) * T + 4 * Mz + 1;    // zMi, zC, b, xo, L, bc
+        if (line == 2) return (4 + 4 + 4 + 2 + 2) * T + 1;         // zMi, zA, zC, b, xo, bc
         return (4 + 2 + 2) * T + 1 + (line ? 8 * Mz : 0);          // Dinv, b, xo, bc (+ L, U)
     case ELDER_K_SPMV: return 108 * Mz + (2 + 2 + 2) * T + 1;        // J, x, y, a, bc
     case ELDER_K_MGRES: return 108 * Mz + (2 + 2 + 2) * T + 1;       // J, x, b, r, bc
     case ELDER_K_RESIDUAL:  // p, c, c_old, R, cval, bc, phi, K
         return 3 * 8 + 16 + 8 + 1 + 16 * cells_per_node;
     case ELDER_K_JACOBIAN:  // J written (Krylov + multigrid copies), Dinv; p, c, bc, phi, K;
-                            // line factors: Dinv, L, U, bc read, zMi, zC written
+                            // line factors: Dinv, L, U, bc read, zMi, zA, zC written
         return 108 * T + 108 * Mz + 4 * Td + 16 + 1 + 16 * cells_per_node +
-               ((line & 1) ? 12 * Td + 8 * Mz + 1 : 0) +
+               ((line & 1) ? 16 * Td + 8 * Mz + 1 : 0) +
                ((line & 2) ? 108 * Mz + 104 * Mz + 8 * Td + 1 : 0);
     }
     return 0.0;
@@ -505,13 +505,12 @@ template <class T> void solver_alloc(elder_ctx* ctx, Solver<T>& sv, int cap)
         sv.Dinv.push_back(dalloc<B4<T>>(nN));
         sv.mem.add(sv.Dinv.back());
         if (G.nz + 1 <= kMaxLine) {
-            sv.zMi.push_back(dalloc<B4<T>>(nN));
-            sv.mem.add(sv.zMi.back());
-            sv.zC.push_back(dalloc<B4<T>>(nN));
-            sv.mem.add(sv.zC.back());
+            for (auto* f : {&sv.zMi, &sv.zA, &sv.zC}) {
+                f->push_back(dalloc<B4<T>>(nN));
+                sv.mem.add(f->back());
+            }
         } else {
-            sv.zMi.push_back(nullptr);
-            sv.zC.push_back(nullptr);
+            for (auto* f : {&sv.zMi, &sv.zA, &sv.zC}) f->push_back(nullptr);
         }
         // the ILU smoother's factors on every smoothed level (the coarsest
         // is solved by its dense inverse)
@@ -591,7 +590,7 @@ void assemble(elder_ctx* ctx, Solver<T>& sv, int S, const double* phi0,
                 launch_line_blocks<T>(G, ph, ctx->bc[0], cellT, nodeT, sv.Dinv[0], sv.Lz, sv.Uz,
                                       sv.vs, mask, mstride, S, st);
                 launch_zline_factor<T, T>(G, sv.Lz, sv.Uz, (size_t)G.N, sv.Dinv[0], ctx->bc[0],
-                                          sv.zMi[0], sv.zC[0], mask, mstride, S, st);
+                                          sv.zMi[0], sv.zA[0], sv.zC[0], mask, mstride, S, st);
                 prof_end(ctx, pi, ELDER_K_JACOBIAN, G, (int)sizeof(T), (int)sizeof(M), n_active,
                          st, 1, true);
                 continue;
@@ -607,8 +606,8 @@ void assemble(elder_ctx* ctx, Solver<T>& sv, int S, const double* phi0,
         if (sv.zMi[l])
             launch_zline_factor<T, M>(G, sv.Jm[l] + slot27(0, 0, -1) * (size_t)G.N,
                                       sv.Jm[l] + slot27(0, 0, 1) * (size_t)G.N, 27 * (size_t)G.N,
-                                      sv.Dinv[l], ctx->bc[l], sv.zMi[l], sv.zC[l], mask, mstride,
-                                      S, st);
+                                      sv.Dinv[l], ctx->bc[l], sv.zMi[l], sv.zA[l], sv.zC[l], mask,
+                                      mstride, S, st);
         // the multicolour ILU factors for the ILU sweeps
         if (sv.F[l])
             launch_ilu_factor<T, M>(G, sv.Jm[l], sv.Dinv[l], ctx->bc[l], sv.F[l], sv.Fd[l],
@@ -689,7 +688,7 @@ void vcycle(elder_ctx* ctx, Solver<T>& sv, int l, const V2<T>* b, V2<T>* out,
     using M = typename Solver<T>::M;
     const int na = ctx->n_active_k;
     const int bs_sm = ctx->bs[ELDER_K_SMOOTH], bs_mr = ctx->bs[ELDER_K_MGRES];
-    const int bs_zl = ctx->bs[ELDER_K_SMOOTH0], spc_zl = ctx->spc[ELDER_K_SMOOTH0];
+    const int bs_zl = ctx->bs[ELDER_K_SMOOTH0];
     // (the transposed residual keeps one sample per CTA: two spill registers)
     const int spc_mr = trans ? 1 : ctx->spc[ELDER_K_MGRES];
     const bool line = ctx->smoother_now == ELDER_SMOOTH_ZLINE && G.nz + 1 <= kMaxLine;
@@ -715,15 +714,8 @@ void vcycle(elder_ctx* ctx, Solver<T>& sv, int l, const V2<T>* b, V2<T>* out,
     };
     // the substitution of a factored z-line sweep
     auto line_solve = [&](const V2<T>* rin, const V2<T>* xin, V2<T>* xout, int mode) {
-        if (mf)
-            launch_zline_apply<T, T>(G, sv.Lz, (size_t)G.N, sv.zMi[l], sv.zC[l], ctx->bc[l], rin,
-                                     xin, xout, ctx->omega_now, mask, KSTRIDE, S, st, mode, bs_zl,
-                                     spc_zl);
-        else
-            launch_zline_apply<T, M>(G, sv.Jm[l] + slot27(0, 0, -1) * (size_t)G.N,
-                                     27 * (size_t)G.N, sv.zMi[l], sv.zC[l], ctx->bc[l], rin, xin,
-                                     xout, ctx->omega_now, mask, KSTRIDE, S, st, mode, bs_zl,
-                                     spc_zl);
+        launch_zline_apply<T>(G, sv.zMi[l], sv.zA[l], sv.zC[l], ctx->bc[l], rin, xin, xout,
+                              ctx->omega_now, mask, KSTRIDE, S, st, mode, bs_zl);
     };
     auto sweep = [&](const V2<T>* xin, V2<T>* xout) {
         if (ilu && xin == nullptr) {
@@ -789,7 +781,7 @@ void autotune(elder_ctx* ctx, Solver<T>& sv, int S, cudaStream_t st)
     const int idx = std::is_same<T, float>::value ? 1 : 0;
     if (ctx->tuned[idx] || !ctx->cfg.autotune) return;
     if (ctx->cfg.autotune == 2) {  // fixed: two samples per CTA, default blocks
-        ctx->spc[ELDER_K_MGRES] = ctx->spc[ELDER_K_SMOOTH0] = 2;
+        ctx->spc[ELDER_K_MGRES] = 2;
         ctx->tuned[idx] = true;
         return;
     }
@@ -836,25 +828,23 @@ void autotune(elder_ctx* ctx, Solver<T>& sv, int S, cudaStream_t st)
             }
         }
     }
-    // (threads per block, samples per CTA) of the multigrid residual and of
-    // the factored z-line sweep from x = 0 (the default V(1,0) cycle's only
-    // sweep); two samples per CTA give a thread two independent stencil rows
-    // or line recursions
+    // (threads per block, samples per CTA) of the multigrid residual (two
+    // samples per CTA give a thread two independent stencil rows) and threads
+    // per block of the factored z-line sweep from x = 0 (the default V(1,0)
+    // cycle's only sweep)
     if (sv.zMi[lt] && G.nz + 1 <= kMaxLine) {
         const int bsm[3] = {kMinBS, kBS, kMaxBS}, bsz[3] = {64, 128, 256};
         for (int c = 0; c < 2; ++c) {
             float best = 1e30f;
-            for (int q = 0; q < 6; ++q) {
+            for (int q = 0; q < (c == 0 ? 6 : 3); ++q) {
                 const int bsq = c == 0 ? bsm[q % 3] : bsz[q % 3], spq = 1 + q / 3;
                 auto run = [&]() {
                     if (c == 0)
                         launch_mg_residual<T, M>(G, sv.Jm[lt], bc, sv.mb[lt], sv.mx[lt],
                                                  sv.mx2[lt], 0, nullptr, 0, S, st, bsq, spq);
                     else
-                        launch_zline_apply<T, M>(G, sv.Jm[lt] + slot27(0, 0, -1) * (size_t)G.N,
-                                                 27 * (size_t)G.N, sv.zMi[lt], sv.zC[lt], bc,
-                                                 sv.mb[lt], nullptr, sv.mx2[lt], 1.0, nullptr, 0, S,
-                                                 st, 1, bsq, spq);
+                        launch_zline_apply<T>(G, sv.zMi[lt], sv.zA[lt], sv.zC[lt], bc, sv.mb[lt],
+                                              nullptr, sv.mx2[lt], 1.0, nullptr, 0, S, st, 1, bsq);
                 };
                 run();
                 CK(cudaEventRecord(e0, st));
@@ -1679,13 +1669,9 @@ void smoother_apply_impl(elder_ctx* ctx, int S, const double* phi, const double*
         launch_smooth<T, M>(G, sv.Jm[0], sv.Dinv[0], ctx->bc[0], bT, nullptr, sv.x, 1.0, trans,
                             nullptr, 0, S, st, kBS);
     } else if (kind == ELDER_SMOOTH_ZLINE) {
-        if (sv.mf_now)
-            launch_zline_apply<T, T>(G, sv.Lz, (size_t)G.N, sv.zMi[0], sv.zC[0], ctx->bc[0], bT,
-                                     nullptr, sv.x, 1.0, nullptr, 0, S, st, 1);
-        else if (!trans && sv.zMi[0])
-            launch_zline_apply<T, M>(G, sv.Jm[0] + slot27(0, 0, -1) * (size_t)G.N,
-                                     27 * (size_t)G.N, sv.zMi[0], sv.zC[0], ctx->bc[0], bT,
-                                     nullptr, sv.x, 1.0, nullptr, 0, S, st, 1);
+        if (!trans && sv.zMi[0])
+            launch_zline_apply<T>(G, sv.zMi[0], sv.zA[0], sv.zC[0], ctx->bc[0], bT, nullptr, sv.x,
+                                  1.0, nullptr, 0, S, st, 1);
         else
             launch_smooth_zline<T, M>(G, sv.Jm[0], sv.Dinv[0], ctx->bc[0], bT, nullptr, sv.x,
                                       1.0, trans, nullptr, 0, S, st, 1);
@@ -1913,7 +1899,7 @@ int elder_create(const elder_config* cfg, elder_ctx** out)
             *q = dalloc<double>(nN);
             ctx->mem.add(*q);
         }
-        for (V2<double>** q : {&ctx->R, &ctx->Rt, &ctx->tmp2}) {
+        for (V2<double>** q : {&ctx->R, &ctx->Rt}) {
             *q = dalloc<V2<double>>(nN);
             ctx->mem.add(*q);
         }

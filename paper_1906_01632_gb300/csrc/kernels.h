@@ -236,22 +236,21 @@ void launch_smooth_zline(const Grid& G, const B4<M>* J, const B4<T>* Dinv, const
                          const V2<T>* b, const V2<T>* x, V2<T>* xo, double omega, int trans,
                          const int* mask, int mstride, int S, cudaStream_t st, int mode);
 
-// Block-LU factors of the vertical lines of a level's (non-transposed)
-// operator, zMi and zC [S][N], and the line sweep that substitutes with
-// them (mode 1: x = 0; mode 2: r is the masked residual of x).  Lines of at
-// most kMaxLine nodes.
+// Factors of the vertical lines of a level's (non-transposed) operator, zMi,
+// zA and zC [S][N], and the line sweep that substitutes with them (mode 1: x =
+// 0; mode 2: r is the masked residual of x).  Lines of at most kMaxLine nodes.
 // The lower and upper line blocks of node n of sample s lie at Lz[s sst + n]
 // and Uz[s sst + n].
 template <class T, class M>
 void launch_zline_factor(const Grid& G, const B4<M>* Lz, const B4<M>* Uz, size_t sst,
-                         const B4<T>* Dinv, const uint8_t* bc, B4<T>* zMi, B4<T>* zC,
+                         const B4<T>* Dinv, const uint8_t* bc, B4<T>* zMi, B4<T>* zA, B4<T>* zC,
                          const int* mask, int mstride, int S, cudaStream_t st);
-// bs threads per block; spc lines of different samples per thread (1 or 2)
-template <class T, class M>
-void launch_zline_apply(const Grid& G, const B4<M>* Lz, size_t sst, const B4<T>* zMi,
-                        const B4<T>* zC, const uint8_t* bc, const V2<T>* r, const V2<T>* x, V2<T>* xo,
+// bs: threads per block (64, 128 or 256)
+template <class T>
+void launch_zline_apply(const Grid& G, const B4<T>* zMi, const B4<T>* zA, const B4<T>* zC,
+                        const uint8_t* bc, const V2<T>* r, const V2<T>* x, V2<T>* xo,
                         double omega, const int* mask, int mstride, int S, cudaStream_t st,
-                        int mode, int bs = 128, int spc = 1);
+                        int mode, int bs = 128);
 
 // Multicolour block ILU_beta(0) smoother.  Colour c = (i&1) + 2(j&1) +
 // 4(k&1); the factors are stored with the node axis in colour-blocked order:

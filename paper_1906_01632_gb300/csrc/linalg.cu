@@ -438,164 +438,251 @@ void launch_smooth_zline(const Grid& G, const B4<M>* J, const B4<T>* Dinv, const
 #undef ELDER_ZL
 }
 
-// Block-LU factors of the vertical lines of a level's operator, once per
-// assembly: for node k of a line, with M_0 = D_0 and M_k = D_k - L_k C_{k-1},
-// zMi = M_k^{-1} and zC = C_k = M_k^{-1} U_k (D the diagonal block, formed
-// as the inverse of the stored inverse Dinv exactly as the line sweep of
-// k_smooth_zline does; L, U the masked vertical line blocks).  Each line
-// sweep then only substitutes: the forward elimination and the inversions
-// leave the per-sweep work.
+// A thread's half of a vertical line: lanes 0-15 of a warp walk 16 neighbouring
+// lines up from the bottom, lanes 16-31 the same lines down from the top, both
+// to the nodes next to the middle one, nz / 2.
+struct LineThread {
+    int col;    // the line (clamped to the last)
+    bool up;    // the half above the middle
+    bool live;  // the line exists
+    int count;  // nodes of this half
+    int end;    // its first node (the line's end)
+    int step;   // to the next node towards the middle
+    __device__ __forceinline__ LineThread(const Grid& G, int sz)
+    {
+        const int c = (blockIdx.x * blockDim.x + threadIdx.x) / 32 * 16 + (threadIdx.x & 15);
+        live = c < sz;
+        col = min(c, sz - 1);
+        up = (threadIdx.x & 16) != 0;
+        const int m = G.nz >> 1;
+        count = up ? G.nz - m : m;
+        end = up ? col + G.nz * sz : col;
+        step = up ? -sz : sz;
+    }
+};
+
+// Factors of the vertical lines of a level's (non-transposed) operator, once
+// per assembly.  A line is eliminated from both ends towards its middle node
+// m = nz / 2: below it, with the diagonal blocks D and the masked line blocks L,
+// U (lower, upper), M_k = D_k - L_k C_{k-1} and C_k = M_k^{-1} U_k, above it M_k =
+// D_k - U_k C_{k+1} and C_k = M_k^{-1} L_k; the middle has both terms.  Stored
+// per node: zMi = M_k^{-1}, zA = M_k^{-1} times the block towards the line's end
+// (what the substitution needs of the previous node) and zC = C_k (the next
+// one); at the middle zA = M_m^{-1} L_m and zC = M_m^{-1} U_m.  Two threads per
+// line, lanes l and l + 16 of a warp, so a line costs half its length in
+// dependent steps and the launch has twice the threads: the serial walk, not the
+// memory, is the time of these kernels on single samples and coarse levels.
+// D is the inverse of the stored inverse Dinv.
 template <class T, class M>
-__global__ void __launch_bounds__(kBS)
+__global__ void __launch_bounds__(128)
     k_zline_factor(Grid G, const B4<M>* __restrict__ Lz, const B4<M>* __restrict__ Uz,
-                   size_t sst, const B4<T>* __restrict__ Dinv, const uint8_t* __restrict__ bc, B4<T>* __restrict__ zMi,
-                   B4<T>* __restrict__ zC, const int* mask, int mstride)
+                   size_t sst, const B4<T>* __restrict__ Dinv, const uint8_t* __restrict__ bc,
+                   B4<T>* __restrict__ zMi, B4<T>* __restrict__ zA, B4<T>* __restrict__ zC,
+                   const int* mask, int mstride)
 {
     const int s = blockIdx.y;
     if (!on(mask, mstride, s)) return;
     const int sz = (G.nx + 1) * (G.ny + 1);
-    const int col = blockIdx.x * blockDim.x + threadIdx.x;
-    if (col >= sz) return;
+    const LineThread lt(G, sz);
     const size_t on_ = (size_t)s * G.N;
-    const B4<M>* Jl = Lz + s * sst;
-    const B4<M>* Ju = Uz + s * sst;
+    const B4<M>* Lo = Lz + s * sst;
+    const B4<M>* Up = Uz + s * sst;
+    // towards the line's end (in) and towards the middle (to)
+    const B4<M>*In = lt.up ? Up : Lo, *To = lt.up ? Lo : Up;
     B4<T> Cp{T(0), T(0), T(0), T(0)};
-    uint8_t bc_prev = 0;
-    for (int k = 0; k <= G.nz; ++k) {
-        const int n = col + k * sz;
-        const uint8_t mk = bc[n];
+    uint8_t mprev = 0;
+    int n = lt.end;
+#pragma unroll 4
+    for (int i = 0; i < lt.count; ++i, n += lt.step) {
+        const uint8_t mk = bc[n], mn = bc[n + lt.step];
         B4<T> Mk = inv2(Dinv[on_ + n]);
-        if (k > 0) {
-            const B4<T> L = mask_block(raw_line_block<T, M, false>(Jl[n]), mk, bc_prev);
-            const B4<T> LC = mul2(L, Cp);
-            Mk.pp -= LC.pp; Mk.pc -= LC.pc; Mk.cp -= LC.cp; Mk.cc -= LC.cc;
-        }
+        const B4<T> A = mask_block(raw_line_block<T, M, false>(In[n]), mk, mprev);
+        const B4<T> B = mask_block(raw_line_block<T, M, false>(To[n]), mk, mn);
+        const bool inner = i > 0;  // (the block of a line's end points nowhere)
+        const B4<T> AC = mul2(A, Cp);
+        if (inner) { Mk.pp -= AC.pp; Mk.pc -= AC.pc; Mk.cp -= AC.cp; Mk.cc -= AC.cc; }
         const B4<T> Mi = inv2(Mk);
-        zMi[on_ + n] = Mi;
-        if (k < G.nz) {
-            const uint8_t bn = bc[n + sz];
-            const B4<T> U = mask_block(raw_line_block<T, M, false>(Ju[n]), mk, bn);
-            Cp = mul2(Mi, U);
+        Cp = mul2(Mi, B);
+        if (lt.live) {
+            zMi[on_ + n] = Mi;
+            zA[on_ + n] = inner ? mul2(Mi, A) : B4<T>{T(0), T(0), T(0), T(0)};
             zC[on_ + n] = Cp;
         }
-        bc_prev = mk;
+        mprev = mk;
     }
+    // the middle node: the other half's last factor crosses the warp
+    const int m = lt.col + (G.nz >> 1) * sz;
+    const bool below = (G.nz >> 1) > 0, above = G.nz > (G.nz >> 1);
+    const B4<T> Co{__shfl_xor_sync(0xffffffffu, Cp.pp, 16), __shfl_xor_sync(0xffffffffu, Cp.pc, 16),
+                   __shfl_xor_sync(0xffffffffu, Cp.cp, 16),
+                   __shfl_xor_sync(0xffffffffu, Cp.cc, 16)};
+    if (lt.up || !lt.live) return;
+    const uint8_t mk = bc[m];
+    B4<T> Mk = inv2(Dinv[on_ + m]);
+    B4<T> L{T(0), T(0), T(0), T(0)}, U = L;
+    if (below) {
+        L = mask_block(raw_line_block<T, M, false>(Lo[m]), mk, bc[m - sz]);
+        const B4<T> LC = mul2(L, Cp);
+        Mk.pp -= LC.pp; Mk.pc -= LC.pc; Mk.cp -= LC.cp; Mk.cc -= LC.cc;
+    }
+    if (above) {
+        U = mask_block(raw_line_block<T, M, false>(Up[m]), mk, bc[m + sz]);
+        const B4<T> UC = mul2(U, Co);
+        Mk.pp -= UC.pp; Mk.pc -= UC.pc; Mk.cp -= UC.cp; Mk.cc -= UC.cc;
+    }
+    const B4<T> Mi = inv2(Mk);
+    zMi[on_ + m] = Mi;
+    zA[on_ + m] = mul2(Mi, L);
+    zC[on_ + m] = mul2(Mi, U);
 }
 
 template <class T, class M>
 void launch_zline_factor(const Grid& G, const B4<M>* Lz, const B4<M>* Uz, size_t sst,
-                         const B4<T>* Dinv, const uint8_t* bc, B4<T>* zMi, B4<T>* zC,
+                         const B4<T>* Dinv, const uint8_t* bc, B4<T>* zMi, B4<T>* zA, B4<T>* zC,
                          const int* mask, int mstride, int S, cudaStream_t st)
 {
     count_launch(1);
-    dim3 grid(nblocks((G.nx + 1) * (G.ny + 1)), S);
-    k_zline_factor<T, M><<<grid, kBS, 0, st>>>(G, Lz, Uz, sst, Dinv, bc, zMi, zC, mask, mstride);
+    // (blocks for every SM, as the sweep)
+    const int lines = (G.nx + 1) * (G.ny + 1);
+    int bs = 128;
+    while (bs > 32 && nblocks(lines, bs / 2) * S < 304) bs /= 2;
+    dim3 grid(nblocks(lines, bs / 2), S);
+    k_zline_factor<T, M><<<grid, bs, 0, st>>>(G, Lz, Uz, sst, Dinv, bc, zMi, zA, zC, mask,
+                                              mstride);
 }
 
-// One damped z-line sweep with the factors of k_zline_factor (the
-// non-transposed operator): forward substitution g_k = zMi_k (r_k - L_k
-// g_{k-1}), g kept in x_out, then back substitution d_k = g_k - zC_k d_{k+1}
-// and x_out = x + omega d (x = 0 in MODE 1; in MODE 2 r is the masked
-// residual b - A x).  One thread per line of SPC samples: the SPC
-// recursions are independent, so their steps overlap (the autotuner picks
-// SPC with the block size); the loads of a node do not depend on the
-// recursion, so unrolled iterations keep several nodes in flight.  An
-// inactive sample's line is read as sample s0's and not written.
-template <class T, class M, int MODE, int SPC>
+// One damped z-line sweep with the factors of k_zline_factor: g_k = zMi_k r_k -
+// zA_k g_{previous} from both ends to the middle, then d_k = g_k - zC_k d_{next} and
+// x_out = x + omega d from the middle out (x = 0 in MODE 1; in MODE 2 r is the
+// masked residual b - A x).  Each of a line's two threads reads a chunk of
+// kZaChunk nodes ahead of the recursion, so that a walk's time is its
+// arithmetic (two fused multiply-adds per node) and not a memory latency per
+// node; g waits in shared memory, [i][thread].  An inactive line is clamped to
+// the last one and not written.
+constexpr int kZaChunk = 4;
+
+template <class T, int MODE>
 __global__ void __launch_bounds__(kBS)
-    k_zline_apply(Grid G, const B4<M>* __restrict__ Lz, size_t sst, const B4<T>* __restrict__ zMi,
+    k_zline_apply(Grid G, const B4<T>* __restrict__ zMi, const B4<T>* __restrict__ zA,
                   const B4<T>* __restrict__ zC, const uint8_t* __restrict__ bc,
-                  const V2<T>* __restrict__ r, const V2<T>* __restrict__ x, V2<T>* xo, T omega,
-                  const int* mask, int mstride, int S)
+                  const V2<T>* __restrict__ r, const V2<T>* __restrict__ x, V2<T>* __restrict__ xo,
+                  T omega, const int* mask, int mstride)
 {
-    const int s0 = blockIdx.y * SPC;
-    bool act[SPC];
-    bool any = false;
-#pragma unroll
-    for (int q = 0; q < SPC; ++q) {
-        act[q] = s0 + q < S && on(mask, mstride, s0 + q);
-        any = any || act[q];
-    }
-    if (!any) return;
-    const int sz = (G.nx + 1) * (G.ny + 1);
-    const int col = blockIdx.x * blockDim.x + threadIdx.x;
-    if (col >= sz) return;
-    size_t on_[SPC], ol_[SPC];
-#pragma unroll
-    for (int q = 0; q < SPC; ++q) {
-        on_[q] = (size_t)(act[q] ? s0 + q : s0) * G.N;
-        ol_[q] = (size_t)(act[q] ? s0 + q : s0) * sst;
-    }
-    V2<T> gp[SPC];
-#pragma unroll
-    for (int q = 0; q < SPC; ++q) gp[q] = V2<T>{T(0), T(0)};
-    uint8_t bc_prev = 0;
-#pragma unroll 4
-    for (int k = 0; k <= G.nz; ++k) {
-        const int n = col + k * sz;
-        const uint8_t mk = bc[n];
-#pragma unroll
-        for (int q = 0; q < SPC; ++q) {
-            const V2<T> bv = r[on_[q] + n];
-            const B4<M> qL = Lz[ol_[q] + (k > 0 ? n : col)];
-            const B4<T> Mi = zMi[on_[q] + n];
-            T rp = (mk & BC_P) ? T(0) : bv.p;
-            T rc = (mk & BC_C) ? T(0) : bv.c;
-            if (k > 0) {
-                const B4<T> L = mask_block(raw_line_block<T, M, false>(qL), mk, bc_prev);
-                rp = fma(-L.pp, gp[q].p, fma(-L.pc, gp[q].c, rp));
-                rc = fma(-L.cp, gp[q].p, fma(-L.cc, gp[q].c, rc));
-            }
-            gp[q] = V2<T>{fma(Mi.pp, rp, Mi.pc * rc), fma(Mi.cp, rp, Mi.cc * rc)};
-            if (act[q]) xo[on_[q] + n] = gp[q];
-        }
-        bc_prev = mk;
-    }
-    V2<T> d[SPC];
-#pragma unroll
-    for (int q = 0; q < SPC; ++q) d[q] = gp[q];
-#pragma unroll 4
-    for (int k = G.nz; k >= 0; --k) {
-        const int n = col + k * sz;
+    extern __shared__ __align__(16) unsigned char za_smem[];
+    V2<T>* gs = reinterpret_cast<V2<T>*>(za_smem) + threadIdx.x;
+    const int s = blockIdx.y;
+    if (!on(mask, mstride, s)) return;
+    const int sz = (G.nx + 1) * (G.ny + 1), bs = blockDim.x;
+    const LineThread lt(G, sz);
+    const size_t on_ = (size_t)s * G.N;
+    zMi += on_; zA += on_; zC += on_; r += on_; xo += on_;
+    if (MODE != 1) x += on_;
+    auto masked = [&](int n) {
+        V2<T> v = r[n];
         const uint8_t m = bc[n];
+        if (m & BC_P) v.p = T(0);
+        if (m & BC_C) v.c = T(0);
+        return v;
+    };
+    B4<T> mi[kZaChunk], za[kZaChunk];
+    V2<T> rv[kZaChunk];
+    auto fetch = [&](int i0) {
 #pragma unroll
-        for (int q = 0; q < SPC; ++q) {
-            if (!act[q]) continue;
-            if (k < G.nz) {
-                const B4<T> C = zC[on_[q] + n];
-                const V2<T> g = xo[on_[q] + n];
-                d[q] = V2<T>{fma(-C.pp, d[q].p, fma(-C.pc, d[q].c, g.p)),
-                             fma(-C.cp, d[q].p, fma(-C.cc, d[q].c, g.c))};
+        for (int q = 0; q < kZaChunk; ++q) {
+            const int n = lt.end + min(i0 + q, max(lt.count - 1, 0)) * lt.step;
+            mi[q] = zMi[n];
+            za[q] = zA[n];
+            rv[q] = masked(n);
+        }
+    };
+    fetch(0);
+    V2<T> g{T(0), T(0)};
+    for (int i0 = 0; i0 < lt.count; i0 += kZaChunk) {
+        B4<T> a[kZaChunk];
+        V2<T> h[kZaChunk];  // zMi r: off the recursion
+#pragma unroll
+        for (int q = 0; q < kZaChunk; ++q) {
+            a[q] = za[q];
+            h[q] = V2<T>{fma(mi[q].pp, rv[q].p, mi[q].pc * rv[q].c),
+                         fma(mi[q].cp, rv[q].p, mi[q].cc * rv[q].c)};
+        }
+        if (i0 + kZaChunk < lt.count) fetch(i0 + kZaChunk);
+#pragma unroll
+        for (int q = 0; q < kZaChunk; ++q) {
+            if (i0 + q < lt.count) {
+                g = V2<T>{fma(-a[q].pp, g.p, fma(-a[q].pc, g.c, h[q].p)),
+                          fma(-a[q].cp, g.p, fma(-a[q].cc, g.c, h[q].c))};
+                gs[(i0 + q) * bs] = g;
             }
-            V2<T> xn{T(0), T(0)};
-            if (MODE != 1) xn = x[on_[q] + n];
-            T op = fma(omega, d[q].p, xn.p), oc = fma(omega, d[q].c, xn.c);
-            if (m & BC_P) op = T(0);
-            if (m & BC_C) oc = T(0);
-            xo[on_[q] + n] = V2<T>{op, oc};
+        }
+    }
+    // backward factors of the nodes next to the middle, and the middle itself
+    const int m = lt.col + (G.nz >> 1) * sz;
+    V2<T> xv[kZaChunk];
+    auto fetch_back = [&](int i1) {
+#pragma unroll
+        for (int q = 0; q < kZaChunk; ++q) {
+            const int n = lt.end + max(i1 - q, 0) * lt.step;
+            mi[q] = zC[n];
+            if (MODE != 1) xv[q] = x[n];
+        }
+    };
+    fetch_back(lt.count - 1);
+    const B4<T> Mm = zMi[m], Am = zA[m], Cm = zC[m];
+    const V2<T> rm = masked(m);
+    const V2<T> o{__shfl_xor_sync(0xffffffffu, g.p, 16), __shfl_xor_sync(0xffffffffu, g.c, 16)};
+    const V2<T> gl = lt.up ? o : g, gu = lt.up ? g : o;
+    V2<T> d;
+    d.p = fma(-Am.pp, gl.p, fma(-Am.pc, gl.c, fma(Mm.pp, rm.p, Mm.pc * rm.c)));
+    d.c = fma(-Am.cp, gl.p, fma(-Am.cc, gl.c, fma(Mm.cp, rm.p, Mm.cc * rm.c)));
+    d.p = fma(-Cm.pp, gu.p, fma(-Cm.pc, gu.c, d.p));
+    d.c = fma(-Cm.cp, gu.p, fma(-Cm.cc, gu.c, d.c));
+    auto put = [&](int n, V2<T> xn) {
+        if (lt.live) xo[n] = V2<T>{fma(omega, d.p, xn.p), fma(omega, d.c, xn.c)};
+    };
+    if (!lt.up) put(m, MODE != 1 ? x[m] : V2<T>{T(0), T(0)});
+    for (int i1 = lt.count - 1; i1 >= 0; i1 -= kZaChunk) {
+        B4<T> c[kZaChunk];
+        V2<T> xn[kZaChunk];
+#pragma unroll
+        for (int q = 0; q < kZaChunk; ++q) {
+            c[q] = mi[q];
+            xn[q] = MODE != 1 ? xv[q] : V2<T>{T(0), T(0)};
+        }
+        if (i1 - kZaChunk >= 0) fetch_back(i1 - kZaChunk);
+#pragma unroll
+        for (int q = 0; q < kZaChunk; ++q) {
+            if (i1 - q >= 0) {
+                const V2<T> gk = gs[(i1 - q) * bs];
+                d = V2<T>{fma(-c[q].pp, d.p, fma(-c[q].pc, d.c, gk.p)),
+                          fma(-c[q].cp, d.p, fma(-c[q].cc, d.c, gk.c))};
+                put(lt.end + (i1 - q) * lt.step, xn[q]);
+            }
         }
     }
 }
 
-template <class T, class M>
-void launch_zline_apply(const Grid& G, const B4<M>* Lz, size_t sst, const B4<T>* zMi,
-                        const B4<T>* zC, const uint8_t* bc, const V2<T>* r, const V2<T>* x, V2<T>* xo,
+template <class T>
+void launch_zline_apply(const Grid& G, const B4<T>* zMi, const B4<T>* zA, const B4<T>* zC,
+                        const uint8_t* bc, const V2<T>* r, const V2<T>* x, V2<T>* xo,
                         double omega, const int* mask, int mstride, int S, cudaStream_t st,
-                        int mode, int bs, int spc)
+                        int mode, int bs)
 {
     count_launch(1);
-    dim3 grid(nblocks((G.nx + 1) * (G.ny + 1), bs), (S + spc - 1) / spc);
-#define ELDER_ZLA(MO, SP)                                                                      \
-    k_zline_apply<T, M, MO, SP><<<grid, bs, 0, st>>>(G, Lz, sst, zMi, zC, bc, r, x, xo,       \
-                                                     T(omega), mask, mstride, S)
-    if (mode == 1) {
-        if (spc == 2) ELDER_ZLA(1, 2);
-        else ELDER_ZLA(1, 1);
-    } else {
-        if (spc == 2) ELDER_ZLA(2, 2);
-        else ELDER_ZLA(2, 1);
-    }
-#undef ELDER_ZLA
+    // at most 64 KiB of waiting values per block, and blocks for every SM
+    // where the grid has the lines (a walk is latency: it gains from an SM's
+    // idle issue slots, not from neighbours)
+    const int half = G.nz - (G.nz >> 1), lines = (G.nx + 1) * (G.ny + 1);
+    while (bs > 32 && (sizeof(V2<T>) * half * bs > 64 * 1024 || nblocks(lines, bs / 2) * S < 304))
+        bs /= 2;
+    dim3 grid(nblocks(lines, bs / 2), S);
+    const size_t smem = sizeof(V2<T>) * half * bs;
+    if (mode == 1)
+        launch_smem(k_zline_apply<T, 1>, grid, bs, smem, st, G, zMi, zA, zC, bc, r, x, xo,
+                    T(omega), mask, mstride);
+    else
+        launch_smem(k_zline_apply<T, 2>, grid, bs, smem, st, G, zMi, zA, zC, bc, r, x, xo,
+                    T(omega), mask, mstride);
 }
 
 // SPC samples per CTA: a thread forms the residual of its node in SPC
@@ -1718,15 +1805,19 @@ ELDER_INST(float)
 #define ELDER_INST_ZLINE(T, M)                                                              \
     template void launch_zline_factor<T, M>(const Grid&, const B4<M>*, const B4<M>*, size_t, \
                                             const B4<T>*, const uint8_t*, B4<T>*, B4<T>*,    \
-                                            const int*, int, int, cudaStream_t);             \
-    template void launch_zline_apply<T, M>(const Grid&, const B4<M>*, size_t, const B4<T>*,  \
-                                           const B4<T>*, const uint8_t*, const V2<T>*,       \
-                                           const V2<T>*, V2<T>*, double, const int*, int,    \
-                                           int, cudaStream_t, int, int, int);
+                                            B4<T>*, const int*, int, int, cudaStream_t);
 ELDER_INST_ZLINE(double, double)
 ELDER_INST_ZLINE(float, __nv_bfloat16)
 ELDER_INST_ZLINE(float, float)
 #undef ELDER_INST_ZLINE
+template void launch_zline_apply<double>(const Grid&, const B4<double>*, const B4<double>*,
+                                         const B4<double>*, const uint8_t*, const V2<double>*,
+                                         const V2<double>*, V2<double>*, double, const int*, int,
+                                         int, cudaStream_t, int, int);
+template void launch_zline_apply<float>(const Grid&, const B4<float>*, const B4<float>*,
+                                        const B4<float>*, const uint8_t*, const V2<float>*,
+                                        const V2<float>*, V2<float>*, double, const int*, int,
+                                        int, cudaStream_t, int, int);
 template void launch_convert<double, float>(const V2<double>*, V2<float>*, size_t, cudaStream_t);
 template void launch_convert<float, double>(const V2<float>*, V2<double>*, size_t, cudaStream_t);
 template void launch_convert<double, double>(const V2<double>*, V2<double>*, size_t, cudaStream_t);
