@@ -452,8 +452,9 @@ void launch_residual(const Grid& G, const Phys& ph, const uint8_t* bc,
 {
     (void)p_old;  // p has no time derivative
     count_launch(2);
-    dim3 gc(nblocks(G.C), S);
-    k_cell_flux<<<gc, kBS, 0, st>>>(G, ph, make_flux_const(G, ph), phi, K, p, c, qf, mask,
+    const int bsc = spread_block(kBS, G.C, S);
+    dim3 gc(nblocks(G.C, bsc), S);
+    k_cell_flux<<<gc, bsc, 0, st>>>(G, ph, make_flux_const(G, ph), phi, K, p, c, qf, mask,
                                     mstride);
     dim3 grid(nblocks(G.N), S);
     const double vsc = G.hx * G.hy * G.hz / (8.0 * ph.dt);
@@ -733,7 +734,8 @@ void launch_jacobian(const Grid& G, const Phys& ph, const uint8_t* bc,
     } else if (inputs == 1) {  // the coefficients are converted already
         launch_node_inputs<T>(G, ph, p, c, nodeT, mask, mstride, S, st);
     }
-    dim3 grid(nblocks(G.N, 128), S);
+    const int bs = spread_block(128, G.N, S);
+    dim3 grid(nblocks(G.N, bs), S);
     // lumped storage volume per unit phi over dt: (h^3 / 8) / dt per cell corner
     const T vscale = T(0.125 * G.hx * G.hy * G.hz / ph.dt);
     const CellGeom cgd = make_geom(G);
@@ -743,7 +745,7 @@ void launch_jacobian(const Grid& G, const Phys& ph, const uint8_t* bc,
         cg.area[d] = T(cgd.area[d]);
     }
     const PhysT<T> pt{T(ph.rho0), T(ph.drho), T(ph.g), T(ph.Dm)};
-    k_jacobian<T, M><<<grid, 128, 0, st>>>(G, pt, cg, bc, cellT, nodeT, JT, JM, Dinv, vscale,
+    k_jacobian<T, M><<<grid, bs, 0, st>>>(G, pt, cg, bc, cellT, nodeT, JT, JM, Dinv, vscale,
                                             mask, mstride);
 }
 template void launch_jacobian<double, double>(const Grid&, const Phys&, const uint8_t*,
@@ -826,7 +828,8 @@ void launch_line_blocks(const Grid& G, const Phys& ph, const uint8_t* bc, const 
         cg.area[d] = T(cgd.area[d]);
     }
     const PhysT<T> pt{T(ph.rho0), T(ph.drho), T(ph.g), T(ph.Dm)};
-    k_line_blocks<T><<<dim3(nblocks(G.N, 128), S), 128, 0, st>>>(
+    const int bs = spread_block(128, G.N, S);
+    k_line_blocks<T><<<dim3(nblocks(G.N, bs), S), bs, 0, st>>>(
         G, pt, cg, bc, cellT, nodeT, Dinv, Lz, Uz, T(0.125 * G.hx * G.hy * G.hz / ph.dt), vs,
         mask, mstride);
 }

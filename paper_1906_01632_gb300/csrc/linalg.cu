@@ -138,6 +138,7 @@ void launch_spmv(const Grid& G, const B4<T>* J, const uint8_t* bc,
                  int mstride, int S, cudaStream_t st, int bs)
 {
     count_launch(1);
+    bs = spread_block(bs, G.N, S);
     dim3 grid(nblocks(G.N, bs), S);
 #define ELDER_SPMV(TR, MO) \
     k_spmv<T, TR, MO><<<grid, bs, 0, st>>>(G, J, bc, x, y, a, partial, mask, mstride)
@@ -544,8 +545,7 @@ void launch_zline_factor(const Grid& G, const B4<M>* Lz, const B4<M>* Uz, size_t
     count_launch(1);
     // (blocks for every SM, as the sweep)
     const int lines = (G.nx + 1) * (G.ny + 1);
-    int bs = 128;
-    while (bs > 32 && nblocks(lines, bs / 2) * S < 304) bs /= 2;
+    const int bs = spread_block(128, 2 * lines, S);
     dim3 grid(nblocks(lines, bs / 2), S);
     k_zline_factor<T, M><<<grid, bs, 0, st>>>(G, Lz, Uz, sst, Dinv, bc, zMi, zA, zC, mask,
                                               mstride);
@@ -673,8 +673,8 @@ void launch_zline_apply(const Grid& G, const B4<T>* zMi, const B4<T>* zA, const 
     // where the grid has the lines (a walk is latency: it gains from an SM's
     // idle issue slots, not from neighbours)
     const int half = G.nz - (G.nz >> 1), lines = (G.nx + 1) * (G.ny + 1);
-    while (bs > 32 && (sizeof(V2<T>) * half * bs > 64 * 1024 || nblocks(lines, bs / 2) * S < 304))
-        bs /= 2;
+    while (bs > 32 && sizeof(V2<T>) * half * bs > 64 * 1024) bs /= 2;
+    bs = spread_block(bs, 2 * lines, S);
     dim3 grid(nblocks(lines, bs / 2), S);
     const size_t smem = sizeof(V2<T>) * half * bs;
     if (mode == 1)
@@ -736,6 +736,7 @@ void launch_mg_residual(const Grid& G, const B4<M>* J, const uint8_t* bc,
                         const int* mask, int mstride, int S, cudaStream_t st, int bs, int spc)
 {
     count_launch(1);
+    bs = spread_block(bs, G.N, (S + spc - 1) / spc);
     dim3 grid(nblocks(G.N, bs), (S + spc - 1) / spc);
 #define ELDER_MGR(TR, SP) \
     k_mg_residual<T, M, TR, SP><<<grid, bs, 0, st>>>(G, J, bc, b, x, r, mask, mstride, S)
@@ -791,8 +792,9 @@ void launch_restrict(const Grid& Gf, const Grid& Gc, const uint8_t* bcc,
                      int S, cudaStream_t st)
 {
     count_launch(1);
-    dim3 grid(nblocks(Gc.N), S);
-    k_restrict<T><<<grid, kBS, 0, st>>>(Gf, Gc, bcc, rf, bco, mask, mstride);
+    const int bs = spread_block(kBS, Gc.N, S);
+    dim3 grid(nblocks(Gc.N, bs), S);
+    k_restrict<T><<<grid, bs, 0, st>>>(Gf, Gc, bcc, rf, bco, mask, mstride);
 }
 
 template <class T>
@@ -841,8 +843,9 @@ void launch_prolong_add(const Grid& Gf, const Grid& Gc, const uint8_t* bcf,
                         int mstride, int S, cudaStream_t st)
 {
     count_launch(1);
-    dim3 grid(nblocks(Gf.N), S);
-    k_prolong_add<T><<<grid, kBS, 0, st>>>(Gf, Gc, bcf, xc, xf, mask, mstride);
+    const int bs = spread_block(kBS, Gf.N, S);
+    dim3 grid(nblocks(Gf.N, bs), S);
+    k_prolong_add<T><<<grid, bs, 0, st>>>(Gf, Gc, bcf, xc, xf, mask, mstride);
 }
 
 // x = A_c^{-1} b on the coarsest grid, one block per sample; the inverse lies
@@ -967,8 +970,9 @@ void launch_bicg_p(const Grid& G, const V2<T>* r, const V2<T>* v, V2<T>* p,
                    const KScal* ks, int S, cudaStream_t st)
 {
     count_launch(1);
-    dim3 grid(nblocks(G.N), S);
-    k_bicg_p<T><<<grid, kBS, 0, st>>>(G.N, r, v, p, ks);
+    const int bs = spread_block(kBS, G.N, S);
+    dim3 grid(nblocks(G.N, bs), S);
+    k_bicg_p<T><<<grid, bs, 0, st>>>(G.N, r, v, p, ks);
 }
 
 template <class T>
@@ -993,8 +997,9 @@ void launch_bicg_s(const Grid& G, const V2<T>* r, const V2<T>* v, V2<T>* s,
 {
     count_launch(1);
     (void)partial;
-    dim3 grid(nblocks(G.N), S);
-    k_bicg_s<T><<<grid, kBS, 0, st>>>(G.N, r, v, s, ks);
+    const int bs = spread_block(kBS, G.N, S);
+    dim3 grid(nblocks(G.N, bs), S);
+    k_bicg_s<T><<<grid, bs, 0, st>>>(G.N, r, v, s, ks);
 }
 
 // Each thread updates kXrNodes consecutive-stride nodes and sums its own
@@ -1265,8 +1270,9 @@ void launch_newton_rhs(const Grid& G, const V2<double>* R, V2<T>* b,
                        const NScal* ns, int S, cudaStream_t st)
 {
     count_launch(1);
-    dim3 grid(nblocks(G.N), S);
-    k_newton_rhs<T><<<grid, kBS, 0, st>>>(G.N, R, b, ns);
+    const int bs = spread_block(kBS, G.N, S);
+    dim3 grid(nblocks(G.N, bs), S);
+    k_newton_rhs<T><<<grid, bs, 0, st>>>(G.N, R, b, ns);
 }
 
 template <class T>
@@ -1406,8 +1412,9 @@ void launch_newton_accept(const Grid& G, double* p, double* c,
                           cudaStream_t st)
 {
     count_launch(1);
-    dim3 grid(nblocks(G.N), S);
-    k_newton_accept<<<grid, kBS, 0, st>>>(G.N, p, c, pt, ct, R, Rt, ns);
+    const int bs = spread_block(kBS, G.N, S);
+    dim3 grid(nblocks(G.N, bs), S);
+    k_newton_accept<<<grid, bs, 0, st>>>(G.N, p, c, pt, ct, R, Rt, ns);
 }
 
 // With inexact linear solves Newton converges linearly: from two
