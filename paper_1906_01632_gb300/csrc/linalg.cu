@@ -439,41 +439,54 @@ void launch_smooth_zline(const Grid& G, const B4<M>* J, const B4<T>* Dinv, const
 #undef ELDER_ZL
 }
 
-// A thread's half of a vertical line: lanes 0-15 of a warp walk 16 neighbouring
-// lines up from the bottom, lanes 16-31 the same lines down from the top, both
-// to the nodes next to the middle one, nz / 2.
-struct LineThread {
+// The lines of the sweeps.  FP32 (kLinePair): two threads per line, lanes 0-15
+// of a warp walk 16 neighbouring lines up from the bottom, lanes 16-31 the same
+// lines down from the top, both to the nodes next to the middle one, nz / 2: a
+// line costs half its length in dependent steps and the launch has twice the
+// threads.  FP64: one thread walks a line from the bottom, in the order of the
+// textbook elimination; the FP64 solver's iterates do not change with the
+// layout of its kernels (gradients of the adjoint switch with the sign of face
+// fluxes that are zero to rounding, which makes another order visible).
+template <class T> constexpr bool kLinePair = std::is_same<T, float>::value;
+
+template <bool PAIR> struct LineThread {
     int col;    // the line (clamped to the last)
     bool up;    // the half above the middle
     bool live;  // the line exists
-    int count;  // nodes of this half
+    int count;  // nodes of this thread's walk
     int end;    // its first node (the line's end)
-    int step;   // to the next node towards the middle
+    int step;   // to the next node
     __device__ __forceinline__ LineThread(const Grid& G, int sz)
     {
-        const int c = (blockIdx.x * blockDim.x + threadIdx.x) / 32 * 16 + (threadIdx.x & 15);
+        const int t = blockIdx.x * blockDim.x + threadIdx.x;
+        const int c = PAIR ? t / 32 * 16 + (t & 15) : t;
         live = c < sz;
         col = min(c, sz - 1);
-        up = (threadIdx.x & 16) != 0;
+        up = PAIR && (t & 16) != 0;
         const int m = G.nz >> 1;
-        count = up ? G.nz - m : m;
+        count = !PAIR ? G.nz + 1 : (up ? G.nz - m : m);
         end = up ? col + G.nz * sz : col;
         step = up ? -sz : sz;
     }
 };
 
+// Threads of a launch over all lines of a level.
+template <class T> inline int line_threads(const Grid& G)
+{
+    return (kLinePair<T> ? 2 : 1) * (G.nx + 1) * (G.ny + 1);
+}
+
 // Factors of the vertical lines of a level's (non-transposed) operator, once
-// per assembly.  A line is eliminated from both ends towards its middle node
+// per assembly.  FP32: a line is eliminated from both ends towards its middle node
 // m = nz / 2: below it, with the diagonal blocks D and the masked line blocks L,
 // U (lower, upper), M_k = D_k - L_k C_{k-1} and C_k = M_k^{-1} U_k, above it M_k =
 // D_k - U_k C_{k+1} and C_k = M_k^{-1} L_k; the middle has both terms.  Stored
 // per node: zMi = M_k^{-1}, zA = M_k^{-1} times the block towards the line's end
 // (what the substitution needs of the previous node) and zC = C_k (the next
-// one); at the middle zA = M_m^{-1} L_m and zC = M_m^{-1} U_m.  Two threads per
-// line, lanes l and l + 16 of a warp, so a line costs half its length in
-// dependent steps and the launch has twice the threads: the serial walk, not the
-// memory, is the time of these kernels on single samples and coarse levels.
-// D is the inverse of the stored inverse Dinv.
+// one); at the middle zA = M_m^{-1} L_m and zC = M_m^{-1} U_m.  FP64: from the
+// bottom to the top, zMi = M_k^{-1}, zA = L_k (masked), zC = C_k.  The serial walk,
+// not the memory, is the time of these kernels on single samples and coarse
+// levels.  D is the inverse of the stored inverse Dinv.
 template <class T, class M>
 __global__ void __launch_bounds__(128)
     k_zline_factor(Grid G, const B4<M>* __restrict__ Lz, const B4<M>* __restrict__ Uz,
@@ -484,7 +497,7 @@ __global__ void __launch_bounds__(128)
     const int s = blockIdx.y;
     if (!on(mask, mstride, s)) return;
     const int sz = (G.nx + 1) * (G.ny + 1);
-    const LineThread lt(G, sz);
+    const LineThread<kLinePair<T>> lt(G, sz);
     const size_t on_ = (size_t)s * G.N;
     const B4<M>* Lo = Lz + s * sst;
     const B4<M>* Up = Uz + s * sst;
@@ -493,6 +506,31 @@ __global__ void __launch_bounds__(128)
     B4<T> Cp{T(0), T(0), T(0), T(0)};
     uint8_t mprev = 0;
     int n = lt.end;
+    if constexpr (!kLinePair<T>) {
+        if (!lt.live) return;
+        zA[on_ + n] = Cp;
+        for (int k = 0; k <= G.nz; ++k) {
+            const int n = lt.col + k * sz;
+            const uint8_t mk = bc[n];
+            B4<T> Mk = inv2(Dinv[on_ + n]);
+            if (k > 0) {
+                const B4<T> L = mask_block(raw_line_block<T, M, false>(Lo[n]), mk, mprev);
+                const B4<T> LC = mul2(L, Cp);
+                Mk.pp -= LC.pp; Mk.pc -= LC.pc; Mk.cp -= LC.cp; Mk.cc -= LC.cc;
+                zA[on_ + n] = L;
+            }
+            const B4<T> Mi = inv2(Mk);
+            zMi[on_ + n] = Mi;
+            if (k < G.nz) {
+                const uint8_t bn = bc[n + sz];
+                const B4<T> U = mask_block(raw_line_block<T, M, false>(Up[n]), mk, bn);
+                Cp = mul2(Mi, U);
+                zC[on_ + n] = Cp;
+            }
+            mprev = mk;
+        }
+        return;
+    }
 #pragma unroll 4
     for (int i = 0; i < lt.count; ++i, n += lt.step) {
         const uint8_t mk = bc[n], mn = bc[n + lt.step];
@@ -544,21 +582,22 @@ void launch_zline_factor(const Grid& G, const B4<M>* Lz, const B4<M>* Uz, size_t
 {
     count_launch(1);
     // (blocks for every SM, as the sweep)
-    const int lines = (G.nx + 1) * (G.ny + 1);
-    const int bs = spread_block(128, 2 * lines, S);
-    dim3 grid(nblocks(lines, bs / 2), S);
+    const int lines = line_threads<T>(G);
+    const int bs = spread_block(128, lines, S);
+    dim3 grid(nblocks(lines, bs), S);
     k_zline_factor<T, M><<<grid, bs, 0, st>>>(G, Lz, Uz, sst, Dinv, bc, zMi, zA, zC, mask,
                                               mstride);
 }
 
 // One damped z-line sweep with the factors of k_zline_factor: g_k = zMi_k r_k -
-// zA_k g_{previous} from both ends to the middle, then d_k = g_k - zC_k d_{next} and
-// x_out = x + omega d from the middle out (x = 0 in MODE 1; in MODE 2 r is the
-// masked residual b - A x).  Each of a line's two threads reads a chunk of
-// kZaChunk nodes ahead of the recursion, so that a walk's time is its
-// arithmetic (two fused multiply-adds per node) and not a memory latency per
-// node; g waits in shared memory, [i][thread].  An inactive line is clamped to
-// the last one and not written.
+// zA_k g_{previous} from both ends to the middle (FP64: g_k = zMi_k (r_k - zA_k
+// g_{k-1}) from the bottom), then d_k = g_k - zC_k d_{next} and x_out = x + omega d
+// back out (x = 0 in MODE 1; in MODE 2 r is the masked residual b - A x).  A
+// thread reads a chunk of kZaChunk nodes ahead of the recursion, so that a
+// walk's time is its arithmetic (two dependent fused multiply-adds per node, FP64
+// four) and not a memory latency per few nodes: 17 to 25 us per launch on single
+// samples before.  g waits in shared memory, [i][thread].  An inactive line is
+// clamped to the last one and not written.
 constexpr int kZaChunk = 4;
 
 template <class T, int MODE>
@@ -573,7 +612,7 @@ __global__ void __launch_bounds__(kBS)
     const int s = blockIdx.y;
     if (!on(mask, mstride, s)) return;
     const int sz = (G.nx + 1) * (G.ny + 1), bs = blockDim.x;
-    const LineThread lt(G, sz);
+    const LineThread<kLinePair<T>> lt(G, sz);
     const size_t on_ = (size_t)s * G.N;
     zMi += on_; zA += on_; zC += on_; r += on_; xo += on_;
     if (MODE != 1) x += on_;
@@ -598,13 +637,18 @@ __global__ void __launch_bounds__(kBS)
     fetch(0);
     V2<T> g{T(0), T(0)};
     for (int i0 = 0; i0 < lt.count; i0 += kZaChunk) {
-        B4<T> a[kZaChunk];
-        V2<T> h[kZaChunk];  // zMi r: off the recursion
+        B4<T> a[kZaChunk], mc[kLinePair<T> ? 1 : kZaChunk];
+        V2<T> h[kZaChunk];  // zMi r: off the recursion (FP64: r)
 #pragma unroll
         for (int q = 0; q < kZaChunk; ++q) {
             a[q] = za[q];
-            h[q] = V2<T>{fma(mi[q].pp, rv[q].p, mi[q].pc * rv[q].c),
-                         fma(mi[q].cp, rv[q].p, mi[q].cc * rv[q].c)};
+            if (kLinePair<T>)
+                h[q] = V2<T>{fma(mi[q].pp, rv[q].p, mi[q].pc * rv[q].c),
+                             fma(mi[q].cp, rv[q].p, mi[q].cc * rv[q].c)};
+            else {
+                h[q] = rv[q];
+                mc[q] = mi[q];
+            }
         }
         if (i0 + kZaChunk < lt.count) fetch(i0 + kZaChunk);
 #pragma unroll
@@ -612,6 +656,9 @@ __global__ void __launch_bounds__(kBS)
             if (i0 + q < lt.count) {
                 g = V2<T>{fma(-a[q].pp, g.p, fma(-a[q].pc, g.c, h[q].p)),
                           fma(-a[q].cp, g.p, fma(-a[q].cc, g.c, h[q].c))};
+                if constexpr (!kLinePair<T>)
+                    g = V2<T>{fma(mc[q].pp, g.p, mc[q].pc * g.c),
+                              fma(mc[q].cp, g.p, mc[q].cc * g.c)};
                 gs[(i0 + q) * bs] = g;
             }
         }
@@ -627,21 +674,31 @@ __global__ void __launch_bounds__(kBS)
             if (MODE != 1) xv[q] = x[n];
         }
     };
-    fetch_back(lt.count - 1);
-    const B4<T> Mm = zMi[m], Am = zA[m], Cm = zC[m];
-    const V2<T> rm = masked(m);
-    const V2<T> o{__shfl_xor_sync(0xffffffffu, g.p, 16), __shfl_xor_sync(0xffffffffu, g.c, 16)};
-    const V2<T> gl = lt.up ? o : g, gu = lt.up ? g : o;
     V2<T> d;
-    d.p = fma(-Am.pp, gl.p, fma(-Am.pc, gl.c, fma(Mm.pp, rm.p, Mm.pc * rm.c)));
-    d.c = fma(-Am.cp, gl.p, fma(-Am.cc, gl.c, fma(Mm.cp, rm.p, Mm.cc * rm.c)));
-    d.p = fma(-Cm.pp, gu.p, fma(-Cm.pc, gu.c, d.p));
-    d.c = fma(-Cm.cp, gu.p, fma(-Cm.cc, gu.c, d.c));
     auto put = [&](int n, V2<T> xn) {
         if (lt.live) xo[n] = V2<T>{fma(omega, d.p, xn.p), fma(omega, d.c, xn.c)};
     };
-    if (!lt.up) put(m, MODE != 1 ? x[m] : V2<T>{T(0), T(0)});
-    for (int i1 = lt.count - 1; i1 >= 0; i1 -= kZaChunk) {
+    // a whole walk ends at its last node, whose g is d
+    int last = lt.count - 1;
+    if constexpr (!kLinePair<T>) {
+        d = g;
+        const int n = lt.end + last * lt.step;
+        put(n, MODE != 1 ? x[n] : V2<T>{T(0), T(0)});
+        --last;
+    }
+    fetch_back(last);
+    if constexpr (kLinePair<T>) {
+        const B4<T> Mm = zMi[m], Am = zA[m], Cm = zC[m];
+        const V2<T> rm = masked(m);
+        const V2<T> o{__shfl_xor_sync(0xffffffffu, g.p, 16), __shfl_xor_sync(0xffffffffu, g.c, 16)};
+        const V2<T> gl = lt.up ? o : g, gu = lt.up ? g : o;
+        d.p = fma(-Am.pp, gl.p, fma(-Am.pc, gl.c, fma(Mm.pp, rm.p, Mm.pc * rm.c)));
+        d.c = fma(-Am.cp, gl.p, fma(-Am.cc, gl.c, fma(Mm.cp, rm.p, Mm.cc * rm.c)));
+        d.p = fma(-Cm.pp, gu.p, fma(-Cm.pc, gu.c, d.p));
+        d.c = fma(-Cm.cp, gu.p, fma(-Cm.cc, gu.c, d.c));
+        if (!lt.up) put(m, MODE != 1 ? x[m] : V2<T>{T(0), T(0)});
+    }
+    for (int i1 = last; i1 >= 0; i1 -= kZaChunk) {
         B4<T> c[kZaChunk];
         V2<T> xn[kZaChunk];
 #pragma unroll
@@ -672,11 +729,11 @@ void launch_zline_apply(const Grid& G, const B4<T>* zMi, const B4<T>* zA, const 
     // at most 64 KiB of waiting values per block, and blocks for every SM
     // where the grid has the lines (a walk is latency: it gains from an SM's
     // idle issue slots, not from neighbours)
-    const int half = G.nz - (G.nz >> 1), lines = (G.nx + 1) * (G.ny + 1);
-    while (bs > 32 && sizeof(V2<T>) * half * bs > 64 * 1024) bs /= 2;
-    bs = spread_block(bs, 2 * lines, S);
-    dim3 grid(nblocks(lines, bs / 2), S);
-    const size_t smem = sizeof(V2<T>) * half * bs;
+    const int walk = kLinePair<T> ? G.nz - (G.nz >> 1) : G.nz + 1, lines = line_threads<T>(G);
+    while (bs > 32 && sizeof(V2<T>) * walk * bs > 64 * 1024) bs /= 2;
+    bs = spread_block(bs, lines, S);
+    dim3 grid(nblocks(lines, bs), S);
+    const size_t smem = sizeof(V2<T>) * walk * bs;
     if (mode == 1)
         launch_smem(k_zline_apply<T, 1>, grid, bs, smem, st, G, zMi, zA, zC, bc, r, x, xo,
                     T(omega), mask, mstride);
@@ -853,7 +910,8 @@ void launch_prolong_add(const Grid& Gf, const Grid& Gc, const uint8_t* bcf,
 // threads share an unknown's sum, each over every kCaSplit-th term, so that a
 // thread has n / kCaSplit independent loads.  The plain product reads a column
 // per step (coalesced over the unknowns); the transposed one a row segment.
-constexpr int kCaSplit = 4;
+// FP64 keeps one running sum per unknown.
+template <class T> constexpr int kCaSplit = std::is_same<T, float>::value ? 4 : 1;
 
 template <class T>
 __global__ void __launch_bounds__(1024)
@@ -869,24 +927,25 @@ __global__ void __launch_bounds__(1024)
     for (int q = threadIdx.x; q < n; q += blockDim.x) bs[q] = bb[q];
     __syncthreads();
     const T* A = Ainv + (size_t)s * n * n;
-    for (int e = threadIdx.x; e < n * kCaSplit; e += blockDim.x) {
+    for (int e = threadIdx.x; e < n * kCaSplit<T>; e += blockDim.x) {
         // plain: consecutive threads take consecutive unknowns; transposed:
         // the kCaSplit threads of an unknown are neighbours
-        const int r = trans ? e / kCaSplit : e % n, c = trans ? e % kCaSplit : e / n;
+        const int r = trans ? e / kCaSplit<T> : e % n, c = trans ? e % kCaSplit<T> : e / n;
         T acc = T(0);
         if (!trans) {
 #pragma unroll 8
-            for (int q = c; q < n; q += kCaSplit) acc = fma(A[(size_t)q * n + r], bs[q], acc);
+            for (int q = c; q < n; q += kCaSplit<T>) acc = fma(A[(size_t)q * n + r], bs[q], acc);
         } else {
 #pragma unroll 8
-            for (int q = c; q < n; q += kCaSplit) acc = fma(A[(size_t)r * n + q], bs[q], acc);
+            for (int q = c; q < n; q += kCaSplit<T>) acc = fma(A[(size_t)r * n + q], bs[q], acc);
         }
         part[c * n + r] = acc;
     }
     __syncthreads();
     T* xx = reinterpret_cast<T*>(x + (size_t)s * (n / 2));
     for (int r = threadIdx.x; r < n; r += blockDim.x)
-        xx[r] = (part[r] + part[n + r]) + (part[2 * n + r] + part[3 * n + r]);
+        xx[r] = kCaSplit<T> == 1 ? part[r]
+                                 : (part[r] + part[n + r]) + (part[2 * n + r] + part[3 * n + r]);
 }
 
 template <class T>
@@ -896,10 +955,10 @@ void launch_coarse_apply(const Grid& G, const double* Ainv, const V2<T>* b,
 {
     count_launch(1);
     const int n = 2 * G.N;
-    const int threads = std::min(1024, (n * kCaSplit + 31) / 32 * 32);
+    const int threads = std::min(1024, (n * kCaSplit<T> + 31) / 32 * 32);
     // the inverse is stored in the solver's arithmetic (CoarseType of its
     // multigrid storage type: FP32 for the mixed solver, FP64 otherwise)
-    launch_smem(k_coarse_apply<T>, dim3(S), threads, sizeof(T) * n * (1 + kCaSplit), st, n,
+    launch_smem(k_coarse_apply<T>, dim3(S), threads, sizeof(T) * n * (1 + kCaSplit<T>), st, n,
                 reinterpret_cast<const T*>(Ainv), b, x, trans, mask, mstride);
 }
 
@@ -1057,32 +1116,34 @@ void launch_bicg_xr(const Grid& G, const V2<T>* ph, const V2<T>* sh,
     k_bicg_xr<T><<<grid, kBS, 0, st>>>(G.N, ph, sh, s, t, rh, x, r, partial, ks);
 }
 
-// Threads of a block that sums nblk partials of one sample: about 8 partials
-// per thread (two batches of 4 loads in flight), at most 1024 threads.  A
-// block's time is its number of dependent load batches: at 256x256x64 the
-// products leave 134 k partials per sum, which 128 threads read in 1,048
-// dependent rounds (391 us); 1024 threads with 4 loads in flight need 33.
-// Two samples of that grid: 302 -> 233 ms per step; one at 128x128x32: 30.3 ->
-// 27.3 ms.
+// Threads of a block that sums nblk partials of one sample.  A block's time
+// is its number of dependent load batches: at 256x256x64 the products leave
+// 134 k partials per sum, which 128 threads read in 1,048 dependent rounds
+// (391 us); 1024 threads with 8 loads in flight need 17.  Two samples of that
+// grid: 302 -> 233 ms per step; one at 128x128x32: 30.3 -> 27.3 ms.  Up to 4096
+// partials 128 threads take at most 4 batches and fix the order of the sums.
 inline int finalize_threads(int nblk)
 {
     int t = 128;
-    while (t < 1024 && 8 * t < nblk) t *= 2;
+    while (nblk > 4096 && t < 1024 && 8 * t < nblk) t *= 2;
     return t;
 }
 
-// This thread's share of sum_q v[q], q < n, in four independent partial sums.
+// This thread's share of sum_q v[q], q < n: one running sum, 8 loads ahead.
 __device__ __forceinline__ double strided_sum(const double* __restrict__ v, int n)
 {
-    double a[4] = {0.0, 0.0, 0.0, 0.0};
+    double a = 0.0;
     const int st = blockDim.x;
     int q = threadIdx.x;
-    for (; q + 3 * st < n; q += 4 * st) {
+    for (; q + 7 * st < n; q += 8 * st) {
+        double b[8];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) a[u] += v[q + u * st];
+        for (int u = 0; u < 8; ++u) b[u] = v[q + u * st];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) a += b[u];
     }
-    for (; q < n; q += st) a[0] += v[q];
-    return (a[0] + a[1]) + (a[2] + a[3]);
+    for (; q < n; q += st) a += v[q];
+    return a;
 }
 
 // This thread's share of the larger of 0 and max_q v[q], q < n.
