@@ -142,6 +142,15 @@ __host__ __device__ inline CellGeom make_geom(const Grid& G)
 // (9,3,3,1)/16.  Output: [S][12][C] records (mass flux m and salt
 // flux F from the edge's lower end A to its upper end B, and the magnitudes
 // of their terms, the round-off scale).
+// FIXED (the mixed solver and elder_residual): the weighted sums of p and c and
+// the porosity sums in fixed point (bits.cuh), each result rounded once; a cell
+// whose values do not fit (infinities, NaN, subnormals) is summed in FP64.  FP64
+// operations per cell 190 -> 82 and per node 75 -> 57: the kernels are bound by
+// the FP64 pipe, and about 1,500 integer operations per cell issue beside it
+// (edge sums in fixed point cost more than they saved: 333 -> 434 us per 64
+// samples).  64 samples at 64x64x16, both kernels: 2070 -> 1196 us; the 256-sample
+// step 151 -> 134 ms.  The FP64 solver keeps the FP64 sums: its iterates do not depend on
+// this form (its residual is 3 % of its step).
 // k_cell_residual: node n sums, for each direction, the 4 quarter faces of
 // its forward edge and of its backward edge (always in the same order, from
 // the edge's lower node, so both ends of an edge use the same value and the
@@ -231,6 +240,60 @@ __device__ __forceinline__ void dir_sums(const R (&p8)[8], const R (&c8)[8], R (
     kron31(cs, sc);
 }
 
+// Largest biased exponent of N values, and whether sums in its unit stay in the
+// normal range (zeros do; subnormals, infinities, NaN and magnitudes below
+// 2^-895 do not: their sums are formed in FP64).
+template <int N>
+__device__ __forceinline__ int top_exponent(const double (&x)[N], bool& fits)
+{
+    int top = 0;
+#pragma unroll
+    for (int L = 0; L < N; ++L) top = max(top, biased_exponent(x[L]));
+    fits = top >= 128 && top <= 1900;
+    if (top == 0) {
+        fits = true;
+#pragma unroll
+        for (int L = 0; L < N; ++L) fits = fits && x[L] == 0.0;
+        top = 1023;
+    }
+    return top;
+}
+
+// Sum of N <= 2^(9 - HEAD) values: in fixed point, else in FP64 in order.
+template <int HEAD, int N> __device__ __forceinline__ double fixed_sum(const double (&x)[N])
+{
+    bool fits;
+    const int top = top_exponent(x, fits);
+    if (fits) {
+        int64_t a = 0;
+#pragma unroll
+        for (int L = 0; L < N; ++L) a += to_fixed<HEAD>(x[L], top);
+        return from_fixed<HEAD>(a, top);
+    }
+    double a = x[0];
+#pragma unroll
+    for (int L = 1; L < N; ++L) a += x[L];
+    return a;
+}
+
+// kron31 in integers
+__device__ __forceinline__ void kron31(const int64_t (&x)[2][2], int64_t (&y)[2][2])
+{
+    int64_t t[2][2];
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+        const int64_t a = x[u][0] + x[u][1];
+        t[u][0] = (x[u][0] << 1) + a;
+        t[u][1] = (x[u][1] << 1) + a;
+    }
+#pragma unroll
+    for (int T_ = 0; T_ < 2; ++T_) {
+        const int64_t a = t[0][T_] + t[1][T_];
+        y[0][T_] = (t[0][T_] << 1) + a;
+        y[1][T_] = (t[1][T_] << 1) + a;
+    }
+}
+
 // the 16x-weighted sums of the direction-D edge differences of p
 template <int D>
 __device__ __forceinline__ void dir_grad(const double (&p8)[8], double (&gp)[2][2])
@@ -242,6 +305,27 @@ __device__ __forceinline__ void dir_grad(const double (&p8)[8], double (&gp)[2][
         for (int v = 0; v < 2; ++v)
             dp[u][v] = p8[corner_of(D, u, v, 1)] - p8[corner_of(D, u, v, 0)];
     kron31(dp, gp);
+}
+
+constexpr int kFluxBS = 128;  // threads per block of k_cell_flux (up to 170 registers)
+
+// The same from the corners in fixed point (to_fixed<kHeadP>, top exponent
+// top).  Differences and weights make 2 x 16: 5 bits above the 57 of a value.
+constexpr int kHeadP = 4;
+template <int D>
+__device__ __forceinline__ void dir_grad_fixed(const int64_t (&p8)[8], int top, double (&gp)[2][2])
+{
+    int64_t dp[2][2], g[2][2];
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+#pragma unroll
+        for (int v = 0; v < 2; ++v)
+            dp[u][v] = p8[corner_of(D, u, v, 1)] - p8[corner_of(D, u, v, 0)];
+    kron31(dp, g);
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+#pragma unroll
+        for (int v = 0; v < 2; ++v) gp[u][v] = from_fixed<kHeadP>(g[u][v], top);
 }
 
 // Z = (W x W x W) x over the cell's corners L = x + 2 y + 4 z: a (3,1) pass
@@ -262,39 +346,61 @@ __device__ __forceinline__ void cube31(const double (&x)[8], double (&Z)[8])
             }
 }
 
+// In fixed point (to_fixed<kHeadC>): Z has 6 bits, the sum of two 7 above the
+// 55 of a value.
+constexpr int kHeadC = 2;
+__device__ __forceinline__ void cube31(const int64_t (&x)[8], int64_t (&Z)[8])
+{
+#pragma unroll
+    for (int L = 0; L < 8; ++L) Z[L] = x[L];
+#pragma unroll
+    for (int d = 0; d < 3; ++d)
+#pragma unroll
+        for (int L = 0; L < 8; ++L)
+            if (!((L >> d) & 1)) {
+                const int H = L | (1 << d);
+                const int64_t a = Z[L] + Z[H];
+                Z[L] = (Z[L] << 1) + a;
+                Z[H] = (Z[H] << 1) + a;
+            }
+}
+
 // Mass flux m and salt flux F of the direction-D quarter face at transverse
 // position (S_, T_), from its edge's lower corner A = corner_of(D, S_, T_, 0)
 // to B; upA: c is upwinded from A.  gp: the direction's 16x-weighted p
-// differences; Zc: the cell's c cube transform; kmuA = K kA_d, dA2 =
-// phi dA2_d.
+// differences; zsum, zdif: sum and difference of the cell's c cube transform at
+// B and A; kmuA = K kA_d, dA2 = phi dA2_d.
 template <int D>
 __device__ __forceinline__ void quarter_face(int S_, int T_, const double (&gp)[2][2],
-                                             const double (&c8)[8], const double (&Zc)[8],
+                                             const double (&c8)[8], double zsum, double zdif,
                                              const Phys& ph, const FluxConst& fc, double kmuA,
                                              double dA2, double& m, double& F, bool& upA)
 {
     const int A = corner_of(D, S_, T_, 0), B = corner_of(D, S_, T_, 1);
-    const double zA = Zc[A], zB = Zc[B];
     // rho = rho0 + drho32 sc16 with 4 sc16 = zA + zB; dA gc16 = dA2 (zB - zA)
-    const double rho = fma(fc.drho128, zA + zB, ph.rho0);
+    const double rho = fma(fc.drho128, zsum, ph.rho0);
     const double G = (D == 2) ? fma(fc.g16h, rho, gp[S_][T_]) : gp[S_][T_];
     m = -(rho * kmuA) * G;
     // upwind end from the sign bit (an integer test)
     upA = __double2hiint(m) >= 0;
     const double cup = upA ? c8[A] : c8[B];
-    F = fma(cup, m, -(rho * dA2) * (zB - zA));
+    F = fma(cup, m, -(rho * dA2) * zdif);
 }
 
-template <int D>
+// Zc and gp of the faces: FIXED from the integer sums (P8 the corners of p, Z8
+// the cube transform of c), else from the FP64 ones.
+template <int D, bool FIXED>
 __device__ __forceinline__ void cell_dir_faces(const double (&p8)[8], const double (&c8)[8],
-                                               const double (&Zc)[8], const float (&pf)[8],
-                                               const float (&cf)[8], const Phys& ph,
-                                               const FluxConst& fc, double Ke, double phie,
-                                               float Kf, float phif, QF* __restrict__ out,
-                                               size_t qs)
+                                               const double (&Zc)[8], const int64_t (&P8)[8],
+                                               const int64_t (&Z8)[8], int topP, int topC,
+                                               const float (&pf)[8], const float (&cf)[8],
+                                               const Phys& ph, const FluxConst& fc, double Ke,
+                                               double phie, float Kf, float phif,
+                                               QF* __restrict__ out, size_t qs)
 {
     double gp[2][2];
-    dir_grad<D>(p8, gp);
+    if (FIXED) dir_grad_fixed<D>(P8, topP, gp);
+    else dir_grad<D>(p8, gp);
     float gpf[2][2], gcf[2][2], scf[2][2];
     dir_sums<float, D>(pf, cf, gpf, gcf, scf);
     const double kmuA = Ke * fc.kA[D], dA2 = phie * fc.dA2[D];
@@ -303,20 +409,24 @@ __device__ __forceinline__ void cell_dir_faces(const double (&p8)[8], const doub
     for (int S_ = 0; S_ < 2; ++S_)
 #pragma unroll
         for (int T_ = 0; T_ < 2; ++T_) {
+            const int A = corner_of(D, S_, T_, 0), B = corner_of(D, S_, T_, 1);
+            const double zsum = FIXED ? from_fixed<kHeadC>(Z8[A] + Z8[B], topC) : Zc[A] + Zc[B];
+            const double zdif = FIXED ? from_fixed<kHeadC>(Z8[B] - Z8[A], topC) : Zc[B] - Zc[A];
             double m, F;
             bool upA;
-            quarter_face<D>(S_, T_, gp, c8, Zc, ph, fc, kmuA, dA2, m, F, upA);
+            quarter_face<D>(S_, T_, gp, c8, zsum, zdif, ph, fc, kmuA, dA2, m, F, upA);
             // rounding scale in FP32: the Darcy flux cancels grad p against rho g
             const float rhof = fmaf(fc.drho32f, scf[S_][T_], fc.rho0f);
             const float mm = rhof * kmuAf *
                              (fabsf(gpf[S_][T_]) + (D == 2 ? fc.g16hf * rhof : 0.0f));
-            const float cupf = upA ? cf[corner_of(D, S_, T_, 0)] : cf[corner_of(D, S_, T_, 1)];
+            const float cupf = upA ? cf[A] : cf[B];
             const float Fm = fmaf(fabsf(cupf), mm, rhof * dAf * fabsf(gcf[S_][T_]));
             out[(size_t)(4 * D + 2 * S_ + T_) * qs] = QF{m, F, mm, Fm};
         }
 }
 
-__global__ void __launch_bounds__(kBS)
+template <bool FIXED>
+__global__ void __launch_bounds__(FIXED ? kFluxBS : kBS, FIXED ? 3 : 2)
     k_cell_flux(Grid G, Phys ph, FluxConst fc, const double* __restrict__ phi,
                 const double* __restrict__ K, const double* __restrict__ p,
                 const double* __restrict__ c, QF* __restrict__ qf, const int* mask, int mstride)
@@ -345,10 +455,32 @@ __global__ void __launch_bounds__(kBS)
     QF* out = qf + (size_t)s * 12 * G.C + e;
     const size_t qs = (size_t)G.C;
     double Zc[8];
-    cube31(c8, Zc);
-    cell_dir_faces<0>(p8, c8, Zc, pf, cf, ph, fc, Ke, phie, Kf, phif, out, qs);
-    cell_dir_faces<1>(p8, c8, Zc, pf, cf, ph, fc, Ke, phie, Kf, phif, out, qs);
-    cell_dir_faces<2>(p8, c8, Zc, pf, cf, ph, fc, Ke, phie, Kf, phif, out, qs);
+    int64_t P8[8], Z8[8];
+    int tp = 0, tc = 0;
+    bool fits = false;
+    if (FIXED) {
+        bool fitp, fitc;
+        tp = top_exponent(p8, fitp);
+        tc = top_exponent(c8, fitc);
+        fits = fitp && fitc;
+    }
+    if (FIXED && fits) {
+        int64_t C8[8];
+#pragma unroll
+        for (int L = 0; L < 8; ++L) {
+            P8[L] = to_fixed<kHeadP>(p8[L], tp);
+            C8[L] = to_fixed<kHeadC>(c8[L], tc);
+        }
+        cube31(C8, Z8);
+        cell_dir_faces<0, true>(p8, c8, Zc, P8, Z8, tp, tc, pf, cf, ph, fc, Ke, phie, Kf, phif, out, qs);
+        cell_dir_faces<1, true>(p8, c8, Zc, P8, Z8, tp, tc, pf, cf, ph, fc, Ke, phie, Kf, phif, out, qs);
+        cell_dir_faces<2, true>(p8, c8, Zc, P8, Z8, tp, tc, pf, cf, ph, fc, Ke, phie, Kf, phif, out, qs);
+    } else {
+        cube31(c8, Zc);
+        cell_dir_faces<0, false>(p8, c8, Zc, P8, Z8, tp, tc, pf, cf, ph, fc, Ke, phie, Kf, phif, out, qs);
+        cell_dir_faces<1, false>(p8, c8, Zc, P8, Z8, tp, tc, pf, cf, ph, fc, Ke, phie, Kf, phif, out, qs);
+        cell_dir_faces<2, false>(p8, c8, Zc, P8, Z8, tp, tc, pf, cf, ph, fc, Ke, phie, Kf, phif, out, qs);
+    }
 }
 
 // Sum of the up to 4 quarter faces of the direction-D edge whose lower node
@@ -378,6 +510,7 @@ __device__ __forceinline__ void edge_sum(const Grid& G, const QF* __restrict__ q
 
 // vsc = |scv| / dt = hx hy hz / (8 dt); the rounding scale (Ap, Ac and the
 // per-block partials of its square) is carried in FP32.
+template <bool FIXED>
 __global__ void __launch_bounds__(kBS)
     k_cell_residual(Grid G, Phys ph, double vsc, const uint8_t* __restrict__ bc,
                     const double* __restrict__ cval, const double* __restrict__ phi,
@@ -387,7 +520,7 @@ __global__ void __launch_bounds__(kBS)
                     double* __restrict__ act, const int* mask, int mstride, float drhof,
                     float rho0f)
 {
-    __shared__ double red[32];
+    __shared__ double red[kBS];
     const int s = blockIdx.y;
     if (!sample_on(mask, mstride, s)) return;
     const size_t on = (size_t)s * G.N, oc = (size_t)s * G.C;
@@ -410,11 +543,23 @@ __global__ void __launch_bounds__(kBS)
         if (k < G.nz) { edge_sum<2>(G, qf, i, j, k, m, F, mm, Fm); Rp += m; Rc += F; Ap += mm; Ac += Fm; }
         if (k > 0) { edge_sum<2>(G, qf, i, j, k - 1, m, F, mm, Fm); Rp -= m; Rc -= F; Ap += mm; Ac += Fm; }
         double phis = 0.0;
+        if (FIXED) {
+            double ps[8];
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            const int ci = i - (q & 1), cj = j - ((q >> 1) & 1), ck = k - (q >> 2);
-            if (ci < 0 || ci >= G.nx || cj < 0 || cj >= G.ny || ck < 0 || ck >= G.nz) continue;
-            phis += __ldg(phi + ci + G.nx * (cj + G.ny * ck));
+            for (int q = 0; q < 8; ++q) {
+                const int ci = i - (q & 1), cj = j - ((q >> 1) & 1), ck = k - (q >> 2);
+                const bool ok =
+                    ci >= 0 && ci < G.nx && cj >= 0 && cj < G.ny && ck >= 0 && ck < G.nz;
+                ps[q] = ok ? __ldg(phi + ci + G.nx * (cj + G.ny * ck)) : 0.0;
+            }
+            phis = fixed_sum<6>(ps);
+        } else {
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                const int ci = i - (q & 1), cj = j - ((q >> 1) & 1), ck = k - (q >> 2);
+                if (ci < 0 || ci >= G.nx || cj < 0 || cj >= G.ny || ck < 0 || ck >= G.nz) continue;
+                phis += __ldg(phi + ci + G.nx * (cj + G.ny * ck));
+            }
         }
         const double vdt = phis * vsc;
         const double cn = c[n], co = c_old[n];
@@ -433,9 +578,22 @@ __global__ void __launch_bounds__(kBS)
         sq = Rp * Rp + Rc * Rc;
         aq = fmaf(Ap, Ap, Ac * Ac);
     }
-    if (partial) {
+    if (partial && !FIXED) {
         const double t = block_sum(sq, red);
         if (threadIdx.x == 0) partial[(size_t)s * gridDim.x + blockIdx.x] = t;
+    }
+    if (partial && FIXED) {
+        // one warp adds the block's values: 13 FP64 operations per block, where
+        // a sum within every warp first takes 10 per thread
+        red[threadIdx.x] = sq;
+        __syncthreads();
+        if (threadIdx.x < 32) {
+            double t = 0.0;
+            for (int q = threadIdx.x; q < blockDim.x; q += 32) t += red[q];
+            t = warp_sum(t);
+            if (threadIdx.x == 0) partial[(size_t)s * gridDim.x + blockIdx.x] = t;
+        }
+        __syncthreads();
     }
     if (act) {
         const float t = block_sum(aq, reinterpret_cast<float*>(red));
@@ -448,19 +606,28 @@ void launch_residual(const Grid& G, const Phys& ph, const uint8_t* bc,
                      const double* p, const double* c, const double* p_old,
                      const double* c_old, V2<double>* R, double* partial,
                      double* act, const int* mask, int mstride, int S,
-                     cudaStream_t st, QF* qf)
+                     cudaStream_t st, QF* qf, bool fixed)
 {
     (void)p_old;  // p has no time derivative
     count_launch(2);
-    const int bsc = spread_block(kBS, G.C, S);
-    dim3 gc(nblocks(G.C, bsc), S);
-    k_cell_flux<<<gc, bsc, 0, st>>>(G, ph, make_flux_const(G, ph), phi, K, p, c, qf, mask,
-                                    mstride);
-    dim3 grid(nblocks(G.N), S);
+    const FluxConst fc = make_flux_const(G, ph);
+    const dim3 grid(nblocks(G.N), S);
     const double vsc = G.hx * G.hy * G.hz / (8.0 * ph.dt);
-    k_cell_residual<<<grid, kBS, 0, st>>>(G, ph, vsc, bc, cval, phi, p, c, c_old, qf, R,
-                                          partial, act, mask, mstride, (float)ph.drho,
-                                          (float)ph.rho0);
+    if (fixed) {
+        const int bs = spread_block(kFluxBS, G.C, S);
+        k_cell_flux<true><<<dim3(nblocks(G.C, bs), S), bs, 0, st>>>(G, ph, fc, phi, K, p, c, qf,
+                                                                    mask, mstride);
+        k_cell_residual<true><<<grid, kBS, 0, st>>>(G, ph, vsc, bc, cval, phi, p, c, c_old, qf, R,
+                                                    partial, act, mask, mstride, (float)ph.drho,
+                                                    (float)ph.rho0);
+    } else {
+        const int bs = spread_block(kBS, G.C, S);
+        k_cell_flux<false><<<dim3(nblocks(G.C, bs), S), bs, 0, st>>>(G, ph, fc, phi, K, p, c, qf,
+                                                                     mask, mstride);
+        k_cell_residual<false><<<grid, kBS, 0, st>>>(G, ph, vsc, bc, cval, phi, p, c, c_old, qf, R,
+                                                     partial, act, mask, mstride, (float)ph.drho,
+                                                     (float)ph.rho0);
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -1751,15 +1918,17 @@ __device__ __forceinline__ double corner_salt_out(const Grid& G, const Phys& ph,
     constexpr int lx = -OX, ly = -OY, lz = -OZ;  // the node's corner of the cell
     double out = 0.0, m, F, gp[2][2];
     bool up;
+    auto zs = [&](int D, int u, int v) { return Zc[corner_of(D, u, v, 0)] + Zc[corner_of(D, u, v, 1)]; };
+    auto zd = [&](int D, int u, int v) { return Zc[corner_of(D, u, v, 1)] - Zc[corner_of(D, u, v, 0)]; };
     // the node is the lower end of the face's edge along D (+F) or the upper (-F)
     dir_grad<0>(p8, gp);
-    quarter_face<0>(ly, lz, gp, c8, Zc, ph, fc, Ke * fc.kA[0], phie * fc.dA2[0], m, F, up);
+    quarter_face<0>(ly, lz, gp, c8, zs(0, ly, lz), zd(0, ly, lz), ph, fc, Ke * fc.kA[0], phie * fc.dA2[0], m, F, up);
     out += lx == 0 ? F : -F;
     dir_grad<1>(p8, gp);
-    quarter_face<1>(lx, lz, gp, c8, Zc, ph, fc, Ke * fc.kA[1], phie * fc.dA2[1], m, F, up);
+    quarter_face<1>(lx, lz, gp, c8, zs(1, lx, lz), zd(1, lx, lz), ph, fc, Ke * fc.kA[1], phie * fc.dA2[1], m, F, up);
     out += ly == 0 ? F : -F;
     dir_grad<2>(p8, gp);
-    quarter_face<2>(lx, ly, gp, c8, Zc, ph, fc, Ke * fc.kA[2], phie * fc.dA2[2], m, F, up);
+    quarter_face<2>(lx, ly, gp, c8, zs(2, lx, ly), zd(2, lx, ly), ph, fc, Ke * fc.kA[2], phie * fc.dA2[2], m, F, up);
     out += lz == 0 ? F : -F;
     return out;
 }

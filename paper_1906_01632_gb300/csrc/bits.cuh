@@ -99,4 +99,57 @@ __host__ __device__ __forceinline__ uint32_t mag_bits(float x)
     return a > 0x7F800000u ? 0x7F800000u : a;
 }
 
+// ---------------------------------------------------------------------------
+// Sums of a few FP64 numbers of one cell in 64-bit integers: the numbers are
+// brought to a common power-of-two unit set by the largest exponent among
+// them, added and weighted exactly, and each result is rounded once.  The unit
+// lies below the last bit of the largest number, so a result is at least as
+// accurate as the same sum in FP64, whose every operation rounds at that scale.
+// Integer operations issue at 64 times the FP64 rate here.
+// ---------------------------------------------------------------------------
+
+// Biased exponent of x (0 for zeros and subnormals, 2047 for infinities, NaN).
+__host__ __device__ __forceinline__ int biased_exponent(double x)
+{
+    return (int)((uint32_t)(bits_of(x) >> 52) & 0x7FFu);
+}
+
+// x in units of 2^(top - 1023 - 52 - HEAD) for biased_exponent(x) <= top < 2047,
+// truncated toward zero (exact where the exponents differ by at most HEAD);
+// subnormals become 0.  Magnitudes stay below 2^(53 + HEAD).
+template <int HEAD> __host__ __device__ __forceinline__ int64_t to_fixed(double x, int top)
+{
+    const uint64_t u = bits_of(x);
+    const int e = (int)((uint32_t)(u >> 52) & 0x7FFu);
+    const int s = top - e < 63 ? top - e : 63;
+    uint64_t m = ((u & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull) << HEAD;
+    m = e == 0 ? 0 : m >> s;
+    const int64_t sign = (int64_t)u >> 63;
+    return ((int64_t)m ^ sign) - sign;
+}
+
+__host__ __device__ __forceinline__ int leading_zeros(uint64_t m)
+{
+#if defined(__CUDA_ARCH__)
+    return __clzll((long long)m);
+#else
+    return __builtin_clzll(m);
+#endif
+}
+
+// v units of to_fixed<HEAD>(., top) as FP64, rounded to nearest (halves away
+// from zero); |v| < 2^63, and 64 <= top <= 1900, so that no result leaves the
+// normal range.
+template <int HEAD> __host__ __device__ __forceinline__ double from_fixed(int64_t v, int top)
+{
+    const uint64_t sign = (uint64_t)v & 0x8000000000000000ull;
+    uint64_t m = v < 0 ? (uint64_t)0 - (uint64_t)v : (uint64_t)v;
+    const int z = leading_zeros(m | 1);
+    m <<= z;  // the leading bit at 63, weight 2^(63 - z) units
+    // 53 bits, rounded; the carry of a full mantissa runs into the exponent
+    const uint64_t r = (m >> 11) + ((m >> 10) & 1);
+    const uint64_t e = (uint64_t)(top - 52 - HEAD + 63 - z - 1);
+    return v == 0 ? 0.0 : double_of(sign | ((e << 52) + r));
+}
+
 }  // namespace elder

@@ -1124,6 +1124,7 @@ bool build_step_graph(elder_ctx* ctx, Solver<T>& sv, int S, const double* phi, c
     const elder_config& cf = ctx->cfg;
     const Grid& G = ctx->grids[0];
     const Phys ph = make_phys(cf, dt);
+    constexpr bool mixed = std::is_same<T, float>::value;
     const size_t nN = (size_t)S * G.N;
     const int nb = ctx->nblk0;
     NScal* ns = ctx->ns;
@@ -1170,7 +1171,7 @@ bool build_step_graph(elder_ctx* ctx, Solver<T>& sv, int S, const double* phi, c
         k_newton_init<<<nblocks(S, 128), 128, 0, cs>>>(ns, S);
         count_launch(1);
         launch_residual(G, ph, ctx->bc[0], ctx->cval, phi, K, p, c, ctx->p_old, ctx->c_old,
-                        ctx->R, ctx->partial, ctx->partial2, nullptr, 0, S, cs, ctx->qf);
+                        ctx->R, ctx->partial, ctx->partial2, nullptr, 0, S, cs, ctx->qf, mixed);
         launch_norm_finalize(ctx->partial, ctx->partial2, nb, ns, 0, S, cs);
         launch_loop_cond(hN, nmask, NSTRIDE, S, cnt + 0, tot + 0, set.newton_maxit, 1, cs);
         CKL();
@@ -1215,7 +1216,7 @@ bool build_step_graph(elder_ctx* ctx, Solver<T>& sv, int S, const double* phi, c
         k1 = g_launches.load();
         launch_residual(G, ph, ctx->bc[0], ctx->cval, phi, K, ctx->pt, ctx->ct, ctx->p_old,
                         ctx->c_old, ctx->Rt, ctx->partial, ctx->partial3, lsmask, NSTRIDE, S, cb2,
-                        ctx->qf);
+                        ctx->qf, mixed);
         launch_norm_finalize(ctx->partial, ctx->partial3, nb, ns, 1, S, cb2);
         launch_newton_ls_finalize(nullptr, ctx->partial2, nb, ns, set.ls_max, S, cb2);
         launch_newton_trial<T>(G, p, c, sv.x, ctx->pt, ctx->ct, ctx->partial2, ns, S, cb2);
@@ -1341,6 +1342,7 @@ int step_impl(elder_ctx* ctx, int S, const double* phi, const double* K, double*
     const elder_config& cf = ctx->cfg;
     const Grid& G = ctx->grids[0];
     const Phys ph = make_phys(cf, dt);
+    constexpr bool mixed = std::is_same<T, float>::value;
     const size_t nN = (size_t)S * G.N;
     const int nb = ctx->nblk0;
     NScal* ns = ctx->ns;
@@ -1378,7 +1380,7 @@ int step_impl(elder_ctx* ctx, int S, const double* phi, const double* K, double*
     CK(cudaMemcpyAsync(ns, ctx->h_ns, sizeof(NScal) * S, cudaMemcpyHostToDevice, st));
     int pi = prof_begin(ctx, st);
     launch_residual(G, ph, ctx->bc[0], ctx->cval, phi, K, p, c, ctx->p_old, ctx->c_old, ctx->R,
-                    ctx->partial, ctx->partial2, nullptr, 0, S, st, ctx->qf);
+                    ctx->partial, ctx->partial2, nullptr, 0, S, st, ctx->qf, mixed);
     prof_end(ctx, pi, ELDER_K_RESIDUAL, G, 8, 8, S, st);
     launch_norm_finalize(ctx->partial, ctx->partial2, nb, ns, 0, S, st);
     CKL();
@@ -1421,7 +1423,7 @@ int step_impl(elder_ctx* ctx, int S, const double* phi, const double* K, double*
             pi = prof_begin(ctx, st);
             launch_residual(G, ph, ctx->bc[0], ctx->cval, phi, K, ctx->pt, ctx->ct, ctx->p_old,
                             ctx->c_old, ctx->Rt, ctx->partial, ctx->partial3, lsmask, NSTRIDE,
-                            S, st, ctx->qf);
+                            S, st, ctx->qf, mixed);
             prof_end(ctx, pi, ELDER_K_RESIDUAL, G, 8, 8, ctx->n_active_ls, st);
             launch_norm_finalize(ctx->partial, ctx->partial3, nb, ns, 1, S, st);
             launch_newton_ls_finalize(nullptr, ctx->partial2, nb, ns, set.ls_max, S, st);
@@ -2005,7 +2007,7 @@ int elder_residual(elder_ctx* ctx, int S, const double* phi, const double* K,
     try {
         launch_residual(ctx->grids[0], make_phys(ctx->cfg, dt), ctx->bc[0], ctx->cval, phi, K,
                         p, c, p_old, c_old, reinterpret_cast<V2<double>*>(R), nullptr, nullptr,
-                        nullptr, 0, S, (cudaStream_t)stream, ctx->qf);
+                        nullptr, 0, S, (cudaStream_t)stream, ctx->qf, true);
         CKL();
     } catch (const Fail& f) {
         return set_error(ctx, f);

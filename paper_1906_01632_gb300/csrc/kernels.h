@@ -101,12 +101,13 @@ void count_launch(int n);
 void set_static_error(const char* msg);
 
 // ---- assembly.cu ---------------------------------------------------------
+// fixed: cell, edge and porosity sums in 64-bit integers (see k_cell_flux)
 void launch_residual(const Grid& G, const Phys& ph, const uint8_t* bc,
                      const double* cval, const double* phi, const double* K,
                      const double* p, const double* c, const double* p_old,
                      const double* c_old, V2<double>* R, double* partial,
                      double* act, const int* mask, int mask_stride, int S,
-                     cudaStream_t st, QF* qf);
+                     cudaStream_t st, QF* qf, bool fixed);
 // Jacobian rows as T (JT) and/or as the multigrid type M (JM), and the inverse
 // interior diagonal blocks (Dinv); null outputs are skipped.  cellT [S][C]
 // and nodeT [S][N] are scratch for the inputs converted to T.
