@@ -5,7 +5,7 @@ Workload: the batched qMC ensemble at 64x64x16 cells (71,825 nodes, 143,650
 unknowns per sample), 256 samples of scrambled-Sobol porosity fields
 phi = 0.1*(1 + 0.3*(xi1 cos(pi x/600) + xi2 cos(pi y/600) + xi3 sin(2 pi
 z/150))/3) with normalised Kozeny-Carman permeability, dt = 1/12 yr, mixed
-precision (bfloat16 multigrid matrices, FP32 Krylov operator and vectors
+precision (bfloat16 coarse multigrid matrices, FP32 matrix-free Krylov operator and vectors
 inside FP64 Newton with FP64 residual and inner products).  One bench step =
 one implicit Euler step of every sample (elder_step_predicted: Newton from
 the quadratic extrapolation of the last states; --predictor 0 uses
@@ -144,7 +144,7 @@ def workload_config(a):
         "parallelism": f"samples sharded, dp{a.gpus}",
         "timed_steps": f"1-{a.steps} of the run from t = 0 (warm-up on a discarded copy)",
         "precision_detail": ("FP64 Newton residual, inner products and state; FP32 Krylov vectors "
-                             "and level-0 Krylov operator; bfloat16 multigrid matrices"
+                             "and level-0 operator (matrix-free); bfloat16 coarse multigrid matrices"
                              if a.precision == "mixed" else "FP64 throughout"),
     }
 
@@ -472,10 +472,19 @@ def run_ours(a):
     tsize = 4 if a.precision == "mixed" else 8
     per_launch_ms = pk["ms"] / max(pk["launches"], 1)
     bytes_per_launch = pk["bytes"] / max(pk["launches"], 1)
-    tr = ncu_traffic(top, a.precision)
+    # the mixed solver's finest level under the z-line smoother stores no matrix
+    mf = a.precision == "mixed" and a.smoother == "zline"
+    mf_top = mf and top in ("spmv", "mg_residual")
+    tr = ncu_traffic(top + "_mf" if mf_top else top, a.precision)
     apk = alu_peaks(E)
     alu = apk["fp64"]
-    if top == "residual" or (top == "jacobian" and a.precision == "fp64"):
+    if mf_top:
+        # matrix-free products: FP32-ALU bound, rated against the FP32 FMA peak
+        # measured on this GPU (mg_residual: with the coarse levels' stored ones)
+        achieved = (pk["flops"] / 1e9) / (pk["ms"] / 1e3) if pk["ms"] > 0 else None
+        bound, peak, unit = "alu", apk["fp32"][0], "GFLOP/s"
+        src = apk["fp32"][1] + "; flops from the per-cell model"
+    elif top == "residual" or (top == "jacobian" and a.precision == "fp64"):
         # FP64-ALU bound (FP64 pipe ~85% busy under ncu): rated against the
         # FP64 FMA peak measured on this GPU
         achieved = (pk["flops"] / 1e9) / (pk["ms"] / 1e3) if pk["ms"] > 0 else None
@@ -491,7 +500,8 @@ def run_ours(a):
                 "traffic": (tr * bytes_per_launch /
                             max(1e-30, E_model_bytes(top, tsize, nx, ny, nz,
                                                      a.smoother != "jacobi",
-                                                     ilu=a.smoother == "ilu"))
+                                                     ilu=a.smoother == "ilu",
+                                                     matrix_free=mf_top))
                             if tr is not None else None),
                 "algorithmic_flops_per_launch": pk["flops"] / max(pk["launches"], 1),
                 "algorithmic_bytes_per_launch": bytes_per_launch, "avg_launch_ms": per_launch_ms,
@@ -505,6 +515,9 @@ def run_ours(a):
     for k, v in classes.items():  # fraction of the class's own bound
         if k == "residual":
             v["bound"], v["frac"] = "fp64 alu", (v["GFLOP/s"] / alu[0] if v["GFLOP/s"] else None)
+        elif mf and k in ("spmv", "mg_residual"):
+            v["bound"] = "fp32 alu"
+            v["frac"] = v["GFLOP/s"] / apk["fp32"][0] if v["GFLOP/s"] else None
         else:
             v["bound"], v["frac"] = "hbm", (v["GB/s"] / hbm_peak if v["GB/s"] else None)
 
@@ -780,10 +793,12 @@ def gpc_timings(E, torch, cfield, stream, Ns=1_000_000, apk=None):
     return res
 
 
-def E_model_bytes(cls, tsize, nx, ny, nz, line=True, ilu=False):
-    """Algorithmic bytes per node of one launch (mirrors the library's model);
-    the mixed path stores the multigrid matrices in bfloat16.  With the z-line
-    smoother the sweep from x = 0 reads the assembly's line factors (zMi, zC),
+def E_model_bytes(cls, tsize, nx, ny, nz, line=True, ilu=False, matrix_free=False):
+    """Algorithmic bytes per node of one launch on a level with a stored matrix
+    (bfloat16 multigrid matrices in the mixed path); matrix_free: the Krylov
+    products and the multigrid residual of the mixed solver's finest level, from
+    the state, the coefficients and the vectors.  With the z-line
+    smoother the sweep from x = 0 reads line factors (zMi, zC),
     the lower line block, b and writes x; the assembly also forms those
     factors (reading Dinv and both line blocks).  With the ILU smoother
     (ilu=True) the sweep from x = 0 reads the 26 factor blocks, the inverse
@@ -793,6 +808,8 @@ def E_model_bytes(cls, tsize, nx, ny, nz, line=True, ilu=False):
     N = (nx + 1) * (ny + 1) * (nz + 1)
     cpn = nx * ny * nz / N
     mz = 2 if tsize == 4 else 8
+    if matrix_free and cls in ("spmv", "mg_residual"):
+        return 8 * tsize + 2 * tsize * cpn + 1
     smooth0 = (12 * tsize + 4 * mz + 1) if line else 8 * tsize + 1
     if ilu:
         smooth0 = 104 * mz + 14 * tsize + 2
