@@ -1128,28 +1128,50 @@ __device__ __forceinline__ void coarse_fill(const Grid& G, const uint8_t* __rest
 }
 
 // Pivot of a step: the largest |col[i]| over the rows not yet used (the lowest
-// of equal ones) and whether another row has an entry.  Called by one warp;
-// used: bit q of lane l is row l + 32 q.
+// of equal ones; a NaN counts as infinity, so that all lanes agree) and whether
+// another row has an entry.  Called by one warp; used: bit q of lane l is row
+// l + 32 q.  On the bit patterns, whose order is that of the absolute values:
+// warp-wide reductions of 32-bit integers instead of five rounds of shuffles
+// and FP64 comparisons on the chain of every step.
+__device__ __forceinline__ unsigned long long gj_key(double a)
+{
+    const unsigned long long b = (unsigned long long)__double_as_longlong(a) & ~(1ull << 63);
+    return min(b, 0x7ff0000000000000ull);
+}
+__device__ __forceinline__ unsigned gj_key(float a)
+{
+    return min(__float_as_uint(a) & 0x7fffffffu, 0x7f800000u);
+}
+// the warp's maximum, for each lane whether its key is equal to it
+__device__ __forceinline__ bool gj_is_max(unsigned long long key)
+{
+    const unsigned hi = (unsigned)(key >> 32), lo = (unsigned)key;
+    // (every lane takes part in both reductions)
+    const bool top = hi == __reduce_max_sync(0xffffffffu, hi);
+    const unsigned low = __reduce_max_sync(0xffffffffu, top ? lo : 0u);
+    return top && lo == low;
+}
+__device__ __forceinline__ bool gj_is_max(unsigned key)
+{
+    return key == __reduce_max_sync(0xffffffffu, key);
+}
+
 template <class R>
 __device__ __forceinline__ int gj_pivot(const R* col, int n, unsigned long long used, bool& other)
 {
+    using K = decltype(gj_key(R(0)));
+    constexpr K unit = sizeof(K) == 8 ? (K)(1ull << 32) : (K)1;
     const int lane = threadIdx.x & 31;
-    R best = R(-1);
-    int bi = 0x7fffffff;  // (a lane without an unused row)
-    int cnt = 0;
+    K best = 0;  // (a lane without an unused row; the others' keys are raised above it)
+    int bi = 0x7fffffff, cnt = 0;
     for (int q = 0, i = lane; i < n; ++q, i += 32) {
-        R a = fabs(col[i]);
-        cnt += a != R(0) ? 1 : 0;
-        if (a != a) a = R(INFINITY);  // a NaN is a pivot like any other: all lanes agree
-        if (!((used >> q) & 1) && a > best) { best = a; bi = i; }
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-        const R ob = __shfl_xor_sync(0xffffffffu, best, o);
-        const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-        if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
+        const K a = gj_key(col[i]);
+        cnt += a != 0 ? 1 : 0;
+        if (!((used >> q) & 1) && a + unit > best) { best = a + unit; bi = i; }
     }
     other = __reduce_add_sync(0xffffffffu, (unsigned)cnt) > 1u;
-    return bi;
+    const bool mine = gj_is_max(best);
+    return (int)__reduce_min_sync(0xffffffffu, mine ? (unsigned)bi : 0x7fffffffu);
 }
 
 // The 16 steps of register slot b0 (a compile-time index, so that v stays in
@@ -1270,9 +1292,13 @@ __global__ void __launch_bounds__(256)
 }
 
 // Any n and type: a cluster of kGjCluster CTAs per sample, each with all rows
-// of its share of the columns.  A step needs one column from its owner (written
-// into every CTA's shared memory, one cluster barrier); the pivot row's entries
-// are local.  SMEM: the share lies in shared memory, else in W.
+// of its share of the columns.  A step needs one column from its owner; the
+// pivot row's entries are local.  The step is a serial chain, not arithmetic
+// (13 of the 100 columns' updates take an SM 0.3 us of FP64 issue at n = 100),
+// so the owner of the next column updates that one first and writes it into
+// every CTA's shared memory, and the cluster barrier's two halves enclose the
+// update of the other columns: 32x32x8 FP64 step (n = 100) 8.23 -> 6.77 ms, with
+// the integer pivot search.  SMEM: the share lies in shared memory, else in W.
 constexpr int kGjCluster = 8;
 
 template <class M, class R, bool SMEM>
@@ -1288,29 +1314,33 @@ __global__ void __cluster_dims__(kGjCluster, 1, 1) __launch_bounds__(256)
     const int rank = (int)cl.block_rank();
     const int n = 2 * G.N, nc = (n + kGjCluster - 1) / kGjCluster;
     const int c0 = min(n, rank * nc), c1 = min(n, c0 + nc), w = c1 - c0;
-    R* col = reinterpret_cast<R*>(gj_smem);  // [2][n], double-buffered by step
-    R* row = col + 2 * n;                    // [nc]
+    // [3][n]: column k is written by its owner while a CTA may still update with
+    // column k - 2; every CTA has arrived for k - 1, so none reads k - 3
+    R* col = reinterpret_cast<R*>(gj_smem);
+    R* row = col + 3 * n;  // [nc]
     R* A = SMEM ? row + nc : W + ((size_t)s * kGjCluster + rank) * n * nc;  // [n][nc]
     int* piv = reinterpret_cast<int*>(row + nc + (SMEM ? (size_t)n * nc : 0));
     int* inv_piv = piv + n;
     __shared__ int sp, sother;
     const int tid = threadIdx.x, lane = tid & 31;
-    const int ti = tid >> 4, tj = tid & 15;
+    // entries of the share in the order of the threads: e = tid, tid + 256, ...
+    const int ws = max(w, 1), i0 = tid / ws, j0 = tid - i0 * ws;
+    const int di = (int)blockDim.x / ws, dj = (int)blockDim.x - di * ws;
     for (int e = tid; e < n * nc; e += blockDim.x) A[e] = R(0);
     __syncthreads();
     coarse_fill<M, R>(G, bc, J + (size_t)s * 27 * G.N, A, nc, c0, c1);
     cl.sync();  // (all CTAs of the cluster run: their shared memory can be written)
+    if (rank == 0) {
+        for (int i = tid; i < n; i += blockDim.x) {
+            const R v = A[(size_t)i * nc];
+            for (int to = 0; to < kGjCluster; ++to) cl.map_shared_rank(col, to)[i] = v;
+        }
+    }
+    asm volatile("barrier.cluster.arrive.release;" ::: "memory");
     unsigned long long used = 0;  // (warp 0)
     for (int k = 0; k < n; ++k) {
-        const int owner = k / nc, buf = (k & 1) * n;
-        if (rank == owner) {
-            for (int e = tid; e < n * kGjCluster; e += blockDim.x) {
-                const int to = e / n, i = e - to * n;
-                cl.map_shared_rank(col, to)[buf + i] = A[(size_t)i * nc + k - c0];
-            }
-        }
-        cl.sync();
-        const R* ck = col + buf;
+        asm volatile("barrier.cluster.wait.acquire;" ::: "memory");  // column k is here
+        const R* ck = col + (k % 3) * n;
         if (tid < 32) {
             bool other;
             const int p = gj_pivot(ck, n, used, other);
@@ -1329,20 +1359,37 @@ __global__ void __cluster_dims__(kGjCluster, 1, 1) __launch_bounds__(256)
             }
         }
         __syncthreads();
-        if (sother) {
-            const int p = sp;
-            for (int i = ti; i < n; i += 16) {
-                if (i == p) continue;
-                const R f = ck[i];
-                for (int j = tj; j < w; j += 16) {
-                    R* q = A + (size_t)i * nc + j;
-                    *q = fma(-f, row[j], c0 + j == k ? R(0) : *q);
+        const int p = sp;
+        const bool other = sother != 0;
+        const int jn = k + 1 - c0;  // the next column, if it is this CTA's
+        const bool mine = k + 1 < n && jn >= 0 && jn < w;
+        if (mine) {
+            const int to_buf = ((k + 1) % 3) * n;
+            for (int i = tid; i < n; i += blockDim.x) {
+                R v = A[(size_t)i * nc + jn];
+                if (other && i != p) {
+                    v = fma(-ck[i], row[jn], v);
+                    A[(size_t)i * nc + jn] = v;
                 }
+                for (int to = 0; to < kGjCluster; ++to)
+                    cl.map_shared_rank(col, to)[to_buf + i] = v;
+            }
+        }
+        if (k + 1 < n) asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+        if (other) {
+            for (int i = i0, j = j0; i < n && w > 0;) {
+                if (i != p && !(mine && j == jn)) {
+                    R* q = A + (size_t)i * nc + j;
+                    *q = fma(-ck[i], row[j], c0 + j == k ? R(0) : *q);
+                }
+                i += di;
+                j += dj;
+                if (j >= w) { j -= w; ++i; }
             }
         }
         __syncthreads();
     }
-    cl.sync();  // no CTA leaves while another may still write to it
+    // (no CTA writes to another after the last column, for which all have waited)
     R* out = Ainv + (size_t)s * n * n;
     for (int e = tid; e < n * w; e += blockDim.x) {
         const int j = e / n, i = e - j * n;
@@ -1356,7 +1403,8 @@ __global__ void __cluster_dims__(kGjCluster, 1, 1) __launch_bounds__(256)
 // that hold the matrix, 0.3 ms on one SM at n = 100.  Against one CTA
 // eliminating [A | I] in shared memory (n = 100) or global memory, the step:
 // 128x64x16 x 4 mixed, n = 180: 62.3 -> 28.4 ms; 128x128x32 mixed, n = 100: 27.3
-// -> 22.3 ms; 32x32x8 FP64, n = 100: 9.9 -> 8.1 ms.
+// -> 22.3 ms; 32x32x8 FP64, n = 100: 9.9 -> 8.1 ms (6.8 with
+// the next column published ahead).
 template <class M>
 void launch_coarse_inverse(const Grid& G, const uint8_t* bc, const B4<M>* J,
                            double* work, double* Ainv, const int* mask,
@@ -1380,7 +1428,7 @@ void launch_coarse_inverse(const Grid& G, const uint8_t* bc, const B4<M>* J,
         }
     }
     const int nc = (n + kGjCluster - 1) / kGjCluster;
-    const size_t base = sizeof(R) * (2 * (size_t)n + nc) + sizeof(int) * 2 * (size_t)n;
+    const size_t base = sizeof(R) * (3 * (size_t)n + nc) + sizeof(int) * 2 * (size_t)n;
     const size_t share = sizeof(R) * (size_t)n * nc;
     R* W = reinterpret_cast<R*>(work);
     if (base + share <= 200 * 1024)
