@@ -30,6 +30,12 @@ constexpr int kGpcMaxDeg = 16;   // largest degree in one variable
 constexpr int kGpcBS = 128;      // threads per block
 constexpr int kGpcProjMax = 256; // threads per block of the projection
 constexpr int kGpcChunk = 128;   // samples per shared-memory chunk (even)
+// Dynamic shared memory that a launch of the projection and of the FP32 count may
+// ask for.  The limits are set to these constants before every launch, never to
+// its own size: they are one value per kernel and device, and another host thread
+// may be about to launch a larger table.
+constexpr int kGpcProjSmem = 224 * 1024;
+constexpr int kGpcExcSmem = 112 * 1024;
 
 // P_0..P_n at x by (k+1) P_{k+1} = (2k+1) x P_k - k P_{k-1} (Appendix A).
 __host__ __device__ inline void legendre_all(int n, double x, double* P)
@@ -891,7 +897,7 @@ int elder_gpc_project(int M, int T, const int32_t* beta, int maxdeg, int Nq, con
     const int TP = round_tp(T);
     // rows of an even length where that fits the shared memory
     auto bytes = [&](int ld) { return sizeof(double) * ((size_t)ld * Nq + 2 * T); };
-    const bool pair = bytes(T + (T & 1)) <= 224 * 1024;
+    const bool pair = bytes(T + (T & 1)) <= kGpcProjSmem;
     const size_t smem = bytes(pair ? T + (T & 1) : T);
     // CTAs of warps per SM that share the groups of 32 nodes most evenly, 8 to
     // 16 warps (the FP64 pipe is full with 8; 16 of up to 128 registers fit, 12
@@ -920,7 +926,7 @@ int elder_gpc_project(int M, int T, const int32_t* beta, int maxdeg, int Nq, con
 #define ELDER_GPC_PROJ2(TPV, PR)                                                                \
     do {                                                                                        \
         e = cudaFuncSetAttribute(k_gpc_project<TPV, PR>,                                        \
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);       \
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, kGpcProjSmem);    \
         if (e == cudaSuccess)                                                                   \
             k_gpc_project<TPV, PR><<<grid, threads, smem, st>>>(M, T, beta, Nq, theta, w, N, u, \
                                                                 coef, mean, var, maxdeg);       \
@@ -1030,10 +1036,12 @@ int elder_gpc_exceed_engine(int engine, int M, int T, const int32_t* beta, int m
                             sizeof(int) * (size_t)T * M;
 #define ELDER_GPC_EXC(TPV, NPTV)                                                                   \
     do {                                                                                           \
-        cudaFuncSetAttribute(k_gpc_exceed<TPV, NPTV, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
-                             (int)smem);                                                           \
-        k_gpc_exceed<TPV, NPTV, 4><<<grid, kGpcBS, smem, st>>>(M, T, beta, N, coef, n_pts, nodes, Ns, \
-                                                            theta, thr, maxdeg, cnt);              \
+        e = cudaFuncSetAttribute(k_gpc_exceed<TPV, NPTV, 4>,                                       \
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, kGpcExcSmem);        \
+        if (e == cudaSuccess)                                                                      \
+            k_gpc_exceed<TPV, NPTV, 4><<<grid, kGpcBS, smem, st>>>(M, T, beta, N, coef, n_pts,     \
+                                                                   nodes, Ns, theta, thr, maxdeg,  \
+                                                                   cnt);                           \
     } while (0)
         switch (TP) {
             case 4: ELDER_GPC_EXC(4, 4); break;

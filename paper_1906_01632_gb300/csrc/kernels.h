@@ -82,16 +82,26 @@ inline int spread_block(int bs, int n, int S)
 // blocks of the BiCGStab x/r update (4 nodes per thread): its partials per sample
 inline int bicg_xr_blocks(int n) { return nblocks((n + 3) / 4); }
 
-// Launch with dynamic shared memory beyond the default limit.  The attribute is
-// set on every such launch (a host call; it does not touch the stream), so it
-// holds on whichever device is current.
+// Dynamic shared memory that any launch of launch_smem may ask for (an SM has 227
+// KiB; the rest is for a kernel's static arrays).
+constexpr int kMostSmem = 200 * 1024;
+
+// Launch with dynamic shared memory of at most kMostSmem.  The limit is one value
+// per kernel and device, shared by all host threads: it is always raised to
+// kMostSmem and never set to a launch's own size, which would reject a larger
+// launch of another thread.  (Set on every launch beyond the default limit: a host
+// call that does not touch the stream, and so holds on whichever device is
+// current.)  A failure stays the calling thread's last error, for the caller's
+// check after its launches.
 template <class... P, class... A>
 void launch_smem(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st,
                  A... args)
 {
-    if (smem > 48 * 1024)
+    if (smem > 48 * 1024 &&
         cudaFuncSetAttribute(reinterpret_cast<const void*>(kernel),
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                             cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             kMostSmem) != cudaSuccess)
+        return;
     kernel<<<grid, threads, smem, st>>>(static_cast<P>(args)...);
 }
 
