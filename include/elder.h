@@ -192,8 +192,15 @@ typedef struct elder_ctx elder_ctx;
 int elder_config_default(elder_config* cfg, int nx, int ny, int nz);
 
 /* Creates a context: validates the grid, builds the multigrid hierarchy and
- * allocates all device workspace for up to cfg->max_samples samples on the
- * current device.  *out receives the handle (NULL on failure). */
+ * allocates the device workspace for up to cfg->max_samples samples on the
+ * current device.  *out receives the handle (NULL on failure).  Two parts of an
+ * ELDER_MIXED context's workspace may come later: its FP64 solver is allocated by
+ * the first call that uses it (a solve with rtol < 1e-6, a gradient, the re-solve
+ * of a failed sample), and under ELDER_SMOOTH_ZLINE the finest level's assembled
+ * rows (648 bytes per node and sample, read by transposed solves and by
+ * elder_smoother_apply of the other kinds or transposed) are allocated last and,
+ * where they do not fit, left to those calls, which then return ELDER_ENOMEM
+ * while there is no room. */
 int elder_create(const elder_config* cfg, elder_ctx** out);
 
 /* Frees the context and its device workspace (NULL is accepted). */

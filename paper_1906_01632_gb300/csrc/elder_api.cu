@@ -60,7 +60,10 @@ template <class X> X* dalloc(size_t n)
 {
     void* p = nullptr;
     if (n == 0) n = 1;
-    CK(cudaMalloc(&p, n * sizeof(X)));
+    const cudaError_t e = cudaMalloc(&p, n * sizeof(X));
+    // (reported here: not left as the last error of a later call's check)
+    if (e != cudaSuccess) cudaGetLastError();
+    CK(e);
     return static_cast<X*>(p);
 }
 
@@ -145,8 +148,8 @@ template <class T> struct Solver : SolverBase {
     using M = typename MgType<T>::type;
     // The mixed solver's finest level needs no stored matrix (mf): products
     // by launch_mf_apply, line blocks Lz, Uz and |scv| / dt (vs) from
-    // launch_line_blocks.  J0 and Jm[0] are then allocated by the first call
-    // that needs the rows (reserve_rows); mf_now: the assembly in use has none.
+    // launch_line_blocks.  J0 and Jm[0] are held for the calls that need the
+    // rows (reserve_rows); mf_now: the assembly in use has none.
     bool mf = false, mf_now = false;
     B4<T> *Lz = nullptr, *Uz = nullptr;
     T* vs = nullptr;
@@ -456,6 +459,19 @@ template <class T> Solver<T>& solver_reserve(elder_ctx* ctx, int cap)
     return *up;
 }
 
+// Room for the finest level's rows of a matrix-free solver, both copies in one
+// allocation: a failed one leaves the solver as it was.
+template <class T> void reserve_rows(elder_ctx* ctx, Solver<T>& sv)
+{
+    if (sv.J0) return;
+    using M = typename Solver<T>::M;
+    const size_t n = (size_t)sv.S * ctx->grids[0].N * 27;
+    unsigned char* q = dalloc<unsigned char>(n * (sizeof(B4<T>) + sizeof(B4<M>)));
+    sv.mem.add(q);
+    sv.J0 = reinterpret_cast<B4<T>*>(q);
+    sv.Jm[0] = reinterpret_cast<B4<M>*>(q + n * sizeof(B4<T>));
+}
+
 template <class T> void solver_alloc(elder_ctx* ctx, Solver<T>& sv, int cap)
 {
     if (sv.S) return;
@@ -540,17 +556,16 @@ template <class T> void solver_alloc(elder_ctx* ctx, Solver<T>& sv, int cap)
     sv.work = dalloc<double>((size_t)S * nc * (nc + 8));  // shares of the elimination
     sv.mem.add(sv.work);
     sv.S = S;
-}
-
-// Room for the finest level's rows of a matrix-free solver.
-template <class T> void reserve_rows(elder_ctx* ctx, Solver<T>& sv)
-{
-    if (sv.J0) return;
-    const size_t n = (size_t)sv.S * ctx->grids[0].N * 27;
-    sv.Jm[0] = dalloc<B4<typename Solver<T>::M>>(n);
-    sv.mem.add(sv.Jm[0]);
-    sv.J0 = dalloc<B4<T>>(n);
-    sv.mem.add(sv.J0);
+    // the rows last, so that a transposed solve or another smoother's application
+    // finds its memory in the middle of a run; a solver without room for them
+    // still steps, and those calls try again
+    if (sv.mf) {
+        try {
+            reserve_rows<T>(ctx, sv);
+        } catch (const Fail& f) {
+            if (f.code != ELDER_ENOMEM) throw;
+        }
+    }
 }
 
 // Re-discretised Jacobians on every level (Section 5.1): level 0 at the
