@@ -21,6 +21,7 @@
 #include <type_traits>
 #include <utility>
 
+#include "cellsums.cuh"
 #include "kernels.h"
 
 namespace elder {
@@ -28,14 +29,6 @@ namespace elder {
 __device__ __forceinline__ bool sample_on(const int* mask, int stride, int s)
 {
     return mask == nullptr || mask[(size_t)s * stride] != 0;
-}
-
-// Local corner L = lx + 2 ly + 4 lz of the edge of direction D with
-// transverse local position (u, v), at end 0 (A) or 1 (B).
-__host__ __device__ constexpr int corner_of(int D, int u, int v, int end)
-{
-    return D == 0 ? (end + 2 * u + 4 * v)
-                  : (D == 1 ? (u + 2 * end + 4 * v) : (u + 2 * v + 4 * end));
 }
 
 // ---------------------------------------------------------------------------
@@ -143,14 +136,17 @@ __host__ __device__ inline CellGeom make_geom(const Grid& G)
 // flux F from the edge's lower end A to its upper end B, and the magnitudes
 // of their terms, the round-off scale).
 // FIXED (the mixed solver and elder_residual): the weighted sums of p and c and
-// the porosity sums in fixed point (bits.cuh), each result rounded once; a cell
-// whose values do not fit (infinities, NaN, subnormals) is summed in FP64.  FP64
-// operations per cell 190 -> 82 and per node 75 -> 57: the kernels are bound by
-// the FP64 pipe, and about 1,500 integer operations per cell issue beside it
-// (edge sums in fixed point cost more than they saved: 333 -> 434 us per 64
-// samples).  64 samples at 64x64x16, both kernels: 2070 -> 1196 us; the 256-sample
-// step 151 -> 134 ms.  The FP64 solver keeps the FP64 sums: its iterates do not depend on
-// this form (its residual is 3 % of its step).
+// the porosity sums in fixed point (cellsums.cuh), each result rounded once; a cell
+// whose values do not fit (infinities, NaN, subnormals; for p also corners of very
+// different magnitude) is summed in FP64.  FP64
+// operations per cell 190 -> 82 (130 where p is summed in FP64) and per node 75 -> 57:
+// the kernels are bound by the FP64 pipe, and about 1,500 integer operations per cell
+// issue beside it (edge sums in fixed point cost more than they saved: 333 -> 434 us
+// per 64 samples).  64 samples at 64x64x16, both kernels: 2070 -> 1196 us with p always
+// in fixed point, 1228 with the topmost of 16 layers in FP64 (rough states; 166 us with
+// and without the choice for a sample at 128x128x32 without such cells); the 256-sample
+// step 151 -> 134 ms.  The FP64 solver keeps the FP64 sums: its iterates do not depend
+// on this form (its residual is 3 % of its step).
 // k_cell_residual: node n sums, for each direction, the 4 quarter faces of
 // its forward edge and of its backward edge (always in the same order, from
 // the edge's lower node, so both ends of an edge use the same value and the
@@ -202,25 +198,6 @@ static FluxConst make_flux_const(const Grid& G, const Phys& ph)
     return f;
 }
 
-// y[S][T] = sum_{u,v} (u == S ? 3 : 1) (v == T ? 3 : 1) x[u][v]
-template <class R>
-__device__ __forceinline__ void kron31(const R (&x)[2][2], R (&y)[2][2])
-{
-    R t[2][2];
-#pragma unroll
-    for (int u = 0; u < 2; ++u) {
-        const R a = x[u][0] + x[u][1];
-        t[u][0] = R(2) * x[u][0] + a;
-        t[u][1] = R(2) * x[u][1] + a;
-    }
-#pragma unroll
-    for (int T_ = 0; T_ < 2; ++T_) {
-        const R a = t[0][T_] + t[1][T_];
-        y[0][T_] = R(2) * t[0][T_] + a;
-        y[1][T_] = R(2) * t[1][T_] + a;
-    }
-}
-
 template <class R, int D>
 __device__ __forceinline__ void dir_sums(const R (&p8)[8], const R (&c8)[8], R (&gp)[2][2],
                                          R (&gc)[2][2], R (&sc)[2][2])
@@ -240,130 +217,7 @@ __device__ __forceinline__ void dir_sums(const R (&p8)[8], const R (&c8)[8], R (
     kron31(cs, sc);
 }
 
-// Largest biased exponent of N values, and whether sums in its unit stay in the
-// normal range (zeros do; subnormals, infinities, NaN and magnitudes below
-// 2^-895 do not: their sums are formed in FP64).
-template <int N>
-__device__ __forceinline__ int top_exponent(const double (&x)[N], bool& fits)
-{
-    int top = 0;
-#pragma unroll
-    for (int L = 0; L < N; ++L) top = max(top, biased_exponent(x[L]));
-    fits = top >= 128 && top <= 1900;
-    if (top == 0) {
-        fits = true;
-#pragma unroll
-        for (int L = 0; L < N; ++L) fits = fits && x[L] == 0.0;
-        top = 1023;
-    }
-    return top;
-}
-
-// Sum of N <= 2^(9 - HEAD) values: in fixed point, else in FP64 in order.
-template <int HEAD, int N> __device__ __forceinline__ double fixed_sum(const double (&x)[N])
-{
-    bool fits;
-    const int top = top_exponent(x, fits);
-    if (fits) {
-        int64_t a = 0;
-#pragma unroll
-        for (int L = 0; L < N; ++L) a += to_fixed<HEAD>(x[L], top);
-        return from_fixed<HEAD>(a, top);
-    }
-    double a = x[0];
-#pragma unroll
-    for (int L = 1; L < N; ++L) a += x[L];
-    return a;
-}
-
-// kron31 in integers
-__device__ __forceinline__ void kron31(const int64_t (&x)[2][2], int64_t (&y)[2][2])
-{
-    int64_t t[2][2];
-#pragma unroll
-    for (int u = 0; u < 2; ++u) {
-        const int64_t a = x[u][0] + x[u][1];
-        t[u][0] = (x[u][0] << 1) + a;
-        t[u][1] = (x[u][1] << 1) + a;
-    }
-#pragma unroll
-    for (int T_ = 0; T_ < 2; ++T_) {
-        const int64_t a = t[0][T_] + t[1][T_];
-        y[0][T_] = (t[0][T_] << 1) + a;
-        y[1][T_] = (t[1][T_] << 1) + a;
-    }
-}
-
-// the 16x-weighted sums of the direction-D edge differences of p
-template <int D>
-__device__ __forceinline__ void dir_grad(const double (&p8)[8], double (&gp)[2][2])
-{
-    double dp[2][2];
-#pragma unroll
-    for (int u = 0; u < 2; ++u)
-#pragma unroll
-        for (int v = 0; v < 2; ++v)
-            dp[u][v] = p8[corner_of(D, u, v, 1)] - p8[corner_of(D, u, v, 0)];
-    kron31(dp, gp);
-}
-
 constexpr int kFluxBS = 128;  // threads per block of k_cell_flux (up to 170 registers)
-
-// The same from the corners in fixed point (to_fixed<kHeadP>, top exponent
-// top).  Differences and weights make 2 x 16: 5 bits above the 57 of a value.
-constexpr int kHeadP = 4;
-template <int D>
-__device__ __forceinline__ void dir_grad_fixed(const int64_t (&p8)[8], int top, double (&gp)[2][2])
-{
-    int64_t dp[2][2], g[2][2];
-#pragma unroll
-    for (int u = 0; u < 2; ++u)
-#pragma unroll
-        for (int v = 0; v < 2; ++v)
-            dp[u][v] = p8[corner_of(D, u, v, 1)] - p8[corner_of(D, u, v, 0)];
-    kron31(dp, g);
-#pragma unroll
-    for (int u = 0; u < 2; ++u)
-#pragma unroll
-        for (int v = 0; v < 2; ++v) gp[u][v] = from_fixed<kHeadP>(g[u][v], top);
-}
-
-// Z = (W x W x W) x over the cell's corners L = x + 2 y + 4 z: a (3,1) pass
-// along each axis, (a, b) -> (2 a + (a + b), 2 b + (a + b))
-__device__ __forceinline__ void cube31(const double (&x)[8], double (&Z)[8])
-{
-#pragma unroll
-    for (int L = 0; L < 8; ++L) Z[L] = x[L];
-#pragma unroll
-    for (int d = 0; d < 3; ++d)
-#pragma unroll
-        for (int L = 0; L < 8; ++L)
-            if (!((L >> d) & 1)) {
-                const int H = L | (1 << d);
-                const double a = Z[L] + Z[H];
-                Z[L] = fma(2.0, Z[L], a);
-                Z[H] = fma(2.0, Z[H], a);
-            }
-}
-
-// In fixed point (to_fixed<kHeadC>): Z has 6 bits, the sum of two 7 above the
-// 55 of a value.
-constexpr int kHeadC = 2;
-__device__ __forceinline__ void cube31(const int64_t (&x)[8], int64_t (&Z)[8])
-{
-#pragma unroll
-    for (int L = 0; L < 8; ++L) Z[L] = x[L];
-#pragma unroll
-    for (int d = 0; d < 3; ++d)
-#pragma unroll
-        for (int L = 0; L < 8; ++L)
-            if (!((L >> d) & 1)) {
-                const int H = L | (1 << d);
-                const int64_t a = Z[L] + Z[H];
-                Z[L] = (Z[L] << 1) + a;
-                Z[H] = (Z[H] << 1) + a;
-            }
-}
 
 // Mass flux m and salt flux F of the direction-D quarter face at transverse
 // position (S_, T_), from its edge's lower corner A = corner_of(D, S_, T_, 0)
@@ -387,9 +241,9 @@ __device__ __forceinline__ void quarter_face(int S_, int T_, const double (&gp)[
     F = fma(cup, m, -(rho * dA2) * zdif);
 }
 
-// Zc and gp of the faces: FIXED from the integer sums (P8 the corners of p, Z8
-// the cube transform of c), else from the FP64 ones.
-template <int D, bool FIXED>
+// gp and the c sums of the faces: FIXP and FIXC from the integer sums (P8 the corners
+// of p, Z8 the cube transform of c), else from the FP64 ones.
+template <int D, bool FIXP, bool FIXC>
 __device__ __forceinline__ void cell_dir_faces(const double (&p8)[8], const double (&c8)[8],
                                                const double (&Zc)[8], const int64_t (&P8)[8],
                                                const int64_t (&Z8)[8], int topP, int topC,
@@ -399,7 +253,7 @@ __device__ __forceinline__ void cell_dir_faces(const double (&p8)[8], const doub
                                                QF* __restrict__ out, size_t qs)
 {
     double gp[2][2];
-    if (FIXED) dir_grad_fixed<D>(P8, topP, gp);
+    if (FIXP) dir_grad_fixed<D>(P8, topP, gp);
     else dir_grad<D>(p8, gp);
     float gpf[2][2], gcf[2][2], scf[2][2];
     dir_sums<float, D>(pf, cf, gpf, gcf, scf);
@@ -410,8 +264,8 @@ __device__ __forceinline__ void cell_dir_faces(const double (&p8)[8], const doub
 #pragma unroll
         for (int T_ = 0; T_ < 2; ++T_) {
             const int A = corner_of(D, S_, T_, 0), B = corner_of(D, S_, T_, 1);
-            const double zsum = FIXED ? from_fixed<kHeadC>(Z8[A] + Z8[B], topC) : Zc[A] + Zc[B];
-            const double zdif = FIXED ? from_fixed<kHeadC>(Z8[B] - Z8[A], topC) : Zc[B] - Zc[A];
+            const double zsum = FIXC ? from_fixed<kHeadC>(Z8[A] + Z8[B], topC) : Zc[A] + Zc[B];
+            const double zdif = FIXC ? from_fixed<kHeadC>(Z8[B] - Z8[A], topC) : Zc[B] - Zc[A];
             double m, F;
             bool upA;
             quarter_face<D>(S_, T_, gp, c8, zsum, zdif, ph, fc, kmuA, dA2, m, F, upA);
@@ -434,6 +288,7 @@ __global__ void __launch_bounds__(FIXED ? kFluxBS : kBS, FIXED ? 3 : 2)
     const int s = blockIdx.y;
     if (!sample_on(mask, mstride, s)) return;
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    const unsigned live = FIXED ? __ballot_sync(0xffffffffu, e < G.C) : 0u;
     if (e >= G.C) return;
     const size_t on = (size_t)s * G.N, oc = (size_t)s * G.C;
     const int ci = e % G.nx, cj = (e / G.nx) % G.ny, ck = e / (G.nx * G.ny);
@@ -457,30 +312,39 @@ __global__ void __launch_bounds__(FIXED ? kFluxBS : kBS, FIXED ? 3 : 2)
     double Zc[8];
     int64_t P8[8], Z8[8];
     int tp = 0, tc = 0;
-    bool fits = false;
+    bool fixp = false, fixc = false;
     if (FIXED) {
-        bool fitp, fitc;
-        tp = top_exponent(p8, fitp);
-        tc = top_exponent(c8, fitc);
-        fits = fitp && fitc;
+        // (the same for a warp's cells, which are neighbours along x: its cells would
+        // otherwise run both forms one after the other)
+        fixp = __all_sync(live, exact_p(p8, tp));
+        tc = top_exponent(c8, fixc);
     }
-    if (FIXED && fits) {
+#define ELDER_FACES(FP, FC)                                                                    \
+    do {                                                                                       \
+        cell_dir_faces<0, FP, FC>(p8, c8, Zc, P8, Z8, tp, tc, pf, cf, ph, fc, Ke, phie, Kf,    \
+                                  phif, out, qs);                                              \
+        cell_dir_faces<1, FP, FC>(p8, c8, Zc, P8, Z8, tp, tc, pf, cf, ph, fc, Ke, phie, Kf,    \
+                                  phif, out, qs);                                              \
+        cell_dir_faces<2, FP, FC>(p8, c8, Zc, P8, Z8, tp, tc, pf, cf, ph, fc, Ke, phie, Kf,    \
+                                  phif, out, qs);                                              \
+    } while (0)
+    if (FIXED && fixc) {
         int64_t C8[8];
 #pragma unroll
-        for (int L = 0; L < 8; ++L) {
-            P8[L] = to_fixed<kHeadP>(p8[L], tp);
-            C8[L] = to_fixed<kHeadC>(c8[L], tc);
-        }
+        for (int L = 0; L < 8; ++L) C8[L] = to_fixed<kHeadC>(c8[L], tc);
         cube31(C8, Z8);
-        cell_dir_faces<0, true>(p8, c8, Zc, P8, Z8, tp, tc, pf, cf, ph, fc, Ke, phie, Kf, phif, out, qs);
-        cell_dir_faces<1, true>(p8, c8, Zc, P8, Z8, tp, tc, pf, cf, ph, fc, Ke, phie, Kf, phif, out, qs);
-        cell_dir_faces<2, true>(p8, c8, Zc, P8, Z8, tp, tc, pf, cf, ph, fc, Ke, phie, Kf, phif, out, qs);
+        if (fixp) {  // (one branch: a choice per direction kept their sums from overlapping)
+#pragma unroll
+            for (int L = 0; L < 8; ++L) P8[L] = to_fixed<kHeadP>(p8[L], tp);
+            ELDER_FACES(true, true);
+        } else {
+            ELDER_FACES(false, true);
+        }
     } else {
         cube31(c8, Zc);
-        cell_dir_faces<0, false>(p8, c8, Zc, P8, Z8, tp, tc, pf, cf, ph, fc, Ke, phie, Kf, phif, out, qs);
-        cell_dir_faces<1, false>(p8, c8, Zc, P8, Z8, tp, tc, pf, cf, ph, fc, Ke, phie, Kf, phif, out, qs);
-        cell_dir_faces<2, false>(p8, c8, Zc, P8, Z8, tp, tc, pf, cf, ph, fc, Ke, phie, Kf, phif, out, qs);
+        ELDER_FACES(false, false);
     }
+#undef ELDER_FACES
 }
 
 // Sum of the up to 4 quarter faces of the direction-D edge whose lower node

@@ -101,10 +101,12 @@ __host__ __device__ __forceinline__ uint32_t mag_bits(float x)
 
 // ---------------------------------------------------------------------------
 // Sums of a few FP64 numbers of one cell in 64-bit integers: the numbers are
-// brought to a common power-of-two unit set by the largest exponent among
-// them, added and weighted exactly, and each result is rounded once.  The unit
-// lies below the last bit of the largest number, so a result is at least as
-// accurate as the same sum in FP64, whose every operation rounds at that scale.
+// brought to a common power-of-two unit set by the largest exponent among them,
+// added and weighted exactly, and each result is rounded once.  A number is cut off
+// below 2^-HEAD of the last bit of the largest: numbers within HEAD binary orders of
+// it are exact, a smaller one is off by less than that unit, however small it is
+// (where FP64 subtracts two small neighbours without error; see cell_p).  FP64
+// rounds every operation by up to half the last bit of its own result.
 // Integer operations issue at 64 times the FP64 rate here.
 // ---------------------------------------------------------------------------
 
