@@ -1671,6 +1671,12 @@ __device__ __forceinline__ bool exceeds(double x, long long tkey)
     return k > tkey && k <= inf;
 }
 
+// neither infinite nor NaN (an integer test)
+__device__ __forceinline__ bool finite_bits(double x)
+{
+    return (__double2hiint(x) & 0x7FF00000) != 0x7FF00000;
+}
+
 template <bool WEIGHTED>
 __global__ void __launch_bounds__(kBS)
     k_moments(int N, int S, double inv, const double* __restrict__ c,
@@ -1724,9 +1730,18 @@ __global__ void __launch_bounds__(kBS)
         P += part[2][r][l];
     }
     if (!WEIGHTED) {  // (inv: 1 / S; all of S fields count exactly 1)
-        S1 *= inv;
-        S2 *= inv;
         P = P == (double)S ? 1.0 : P * inv;
+        if (finite_bits(S1) && finite_bits(S2)) {
+            S1 *= inv;
+            S2 *= inv;
+        } else {  // beyond the range before the weight (or not finite): weigh every term
+            S1 = S2 = 0.0;
+            for (int s = 0; s < S; ++s) {
+                const double d = c[(size_t)s * N + n] - c0, wd = inv * d;
+                S1 += wd;
+                S2 = fma(wd, d, S2);
+            }
+        }
     }
     const double m = fma(c0, W, S1);
     const double dm = m - c0;
