@@ -396,8 +396,10 @@ int elder_launch_count(int64_t* launches);
  * candidates [samples per CTA 1, 2][threads ascending], 0 when not tuned (the
  * sweep has one line set per CTA: the last 3 are 0);
  * for the other classes 0.  Timed on the first step of a context (3
- * launches after a warm-up, CUDA events) on its level-0 operator with all
- * samples active.  Host outputs; any may be NULL. */
+ * launches after a warm-up, CUDA events) with all samples active: the
+ * residual on its finest stored operator (level 0; level 1 where the mixed
+ * solver's finest level is matrix-free, on which the residual kernel does not
+ * run), the sweep on level 0.  Host outputs; any may be NULL. */
 int elder_autotune_choice(const elder_ctx* ctx, int kernel_class, int* threads_per_block,
                           int* samples_per_cta, float* ms);
 

@@ -247,7 +247,7 @@ struct elder_ctx {
     int nblk0 = 0;
     // threads per block of the autotuned kernel classes (indexed by ELDER_K_*)
     int bs[ELDER_K_CLASSES] = {kBS, kBS, kBS, kBS, kBS, 128};
-    // samples per CTA of the multigrid residual and the z-line sweep
+    // samples per CTA of the multigrid residual (1 in the other classes)
     int spc[ELDER_K_CLASSES] = {1, 1, 1, 1, 1, 1};
     // the (threads per block, samples per CTA) candidates' ms per launch of
     // the multigrid residual [0] and the z-line sweep [1]
@@ -786,10 +786,11 @@ void vcycle(elder_ctx* ctx, Solver<T>& sv, int l, const V2<T>* b, V2<T>* out,
                                        cudaMemcpyDeviceToDevice, st));
 }
 
-// Autotuner: threads per block of the three J-streaming kernel classes,
-// chosen once per context and precision by timing every candidate (CUDA
-// events, 3 launches after a warm-up) on the finest stored
-// operator of a step's first assembly with all S samples active.
+// Autotuner: threads per block of the three J-streaming kernel classes and of the
+// z-line sweep, chosen once per context and precision by timing every candidate
+// (CUDA events, 3 launches after a warm-up) on a step's first assembly with all S
+// samples active: the streaming kernels on the finest stored operator (level 1
+// under a matrix-free finest level, which they do not run on), the sweep on level 0.
 template <class T>
 void autotune(elder_ctx* ctx, Solver<T>& sv, int S, cudaStream_t st)
 {
@@ -844,10 +845,12 @@ void autotune(elder_ctx* ctx, Solver<T>& sv, int S, cudaStream_t st)
         }
     }
     // (threads per block, samples per CTA) of the multigrid residual (two
-    // samples per CTA give a thread two independent stencil rows) and threads
-    // per block of the factored z-line sweep from x = 0 (the default V(1,0)
-    // cycle's only sweep)
-    if (sv.zMi[lt] && G.nz + 1 <= kMaxLine) {
+    // samples per CTA give a thread two independent stencil rows), on the same
+    // level, and threads per block of the factored z-line sweep from x = 0 (the
+    // default V(1,0) cycle's only sweep) on level 0, where most of its time is
+    if (sv.zMi[0] && ctx->grids[0].nz + 1 <= kMaxLine) {
+        const Grid& G0 = ctx->grids[0];
+        if (lt != 0) CK(cudaMemsetAsync(sv.mb[0], 0, sizeof(V2<T>) * (size_t)S * G0.N, st));
         const int bsm[3] = {kMinBS, kBS, kMaxBS}, bsz[3] = {64, 128, 256};
         for (int c = 0; c < 2; ++c) {
             float best = 1e30f;
@@ -858,8 +861,9 @@ void autotune(elder_ctx* ctx, Solver<T>& sv, int S, cudaStream_t st)
                         launch_mg_residual<T, M>(G, sv.Jm[lt], bc, sv.mb[lt], sv.mx[lt],
                                                  sv.mx2[lt], 0, nullptr, 0, S, st, bsq, spq);
                     else
-                        launch_zline_apply<T>(G, sv.zMi[lt], sv.zA[lt], sv.zC[lt], bc, sv.mb[lt],
-                                              nullptr, sv.mx2[lt], 1.0, nullptr, 0, S, st, 1, bsq);
+                        launch_zline_apply<T>(G0, sv.zMi[0], sv.zA[0], sv.zC[0], ctx->bc[0],
+                                              sv.mb[0], nullptr, sv.mx2[0], 1.0, nullptr, 0, S,
+                                              st, 1, bsq);
                 };
                 run();
                 CK(cudaEventRecord(e0, st));
