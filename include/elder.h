@@ -374,10 +374,12 @@ int elder_profile(elder_ctx* ctx, int on);
  *   JACOBIAN 40 T + 18 + 2 T C/N   SMOOTH 26 T + 2 T C/N + 2.
  * (the Jacobian writes the Krylov and the multigrid copies of J and the
  * inverse diagonal blocks; the residual reads p, c, c_old, phi, K and writes
- * R).  Flops: the FP64 residual counts 266 C/N + 75 of its factored face
- * form, the stencil products 216 + their vector terms, the matrix-free ones
- * 512 C/N + 29.  Any output pointer
- * may be NULL.  Host outputs. */
+ * R).  Flops, of the arithmetic that runs in floating point: the FP64 residual
+ * 266 C/N + 75 of its factored face form, with the mixed solver's sums in
+ * 64-bit integers 110 C/N + 67; the assembly 2890 per full row, 1722 for the
+ * line blocks of a matrix-free level; the stencil products 216 + their vector
+ * terms, the matrix-free ones 512 C/N + 29.  Any output pointer may be NULL.
+ * Host outputs. */
 int elder_profile_read(const elder_ctx* ctx, int kernel_class,
                        int64_t* launches, double* ms, double* bytes,
                        double* flops);

@@ -317,9 +317,9 @@ double model_bytes(int cls, int T, int Mz, const Grid& G, int line, bool mf)
     // scratch vector written, read and written again, x_out, bc twice).
     // line (JACOBIAN): bit 0 with the line factorisation, bit 1 with the ILU
     // factorisation (J, Dinv and bc read, the factors written).
-    // mf: the mixed solver's finest level, whose operator is not stored
-    // (products from the state (p', c) and the coefficients (phi, K/mu), line
-    // blocks in T).
+    // mf: the mixed solver's form on its finest level, whose operator is not
+    // stored (products from the state (p', c) and the coefficients (phi, K/mu),
+    // line blocks in T); the residual moves the same bytes.
     const double cells_per_node = (double)G.C / G.N;
     const int Td = T ? T : Mz;
     const double mf_inputs = 2 * T + 2 * T * cells_per_node;
@@ -375,9 +375,15 @@ double model_flops(int cls, const Grid& G, bool mf)
         // c values and 8 (+2 on vertical edges) for rho, m, F (128); 6 for
         // the coefficients: 266.  Per node: 36 edge sums, 10 edge
         // accumulations, 8 porosity sums and 21 for storage and the squared
-        // norm: 75.
-        return 266 * cells_per_node + 75;
-    case ELDER_K_JACOBIAN: return 24 * (54 + 66) + 10;
+        // norm: 75.  In the mixed solver (mf) the sums of p and c, the sums and
+        // differences of the weighted c values (156) and the porosity sums are
+        // 64-bit integer operations: 110 and 67 FP64 flops remain (a warp of
+        // cells of very different p: 72 more).
+        return mf ? 110 * cells_per_node + 67 : 266 * cells_per_node + 75;
+    case ELDER_K_JACOBIAN:
+        // 24 faces of 54 for their values; 66 for all entries of the row, or (mf)
+        // 16 and the upwind term for the two corners on the node's vertical line
+        return mf ? 24 * (54 + 16) + 32 + 10 : 24 * (54 + 66) + 10;
     }
     return 0.0;
 }
@@ -1400,7 +1406,7 @@ int step_impl(elder_ctx* ctx, int S, const double* phi, const double* K, double*
     int pi = prof_begin(ctx, st);
     launch_residual(G, ph, ctx->bc[0], ctx->cval, phi, K, p, c, ctx->p_old, ctx->c_old, ctx->R,
                     ctx->partial, ctx->partial2, nullptr, 0, S, st, ctx->qf, mixed);
-    prof_end(ctx, pi, ELDER_K_RESIDUAL, G, 8, 8, S, st);
+    prof_end(ctx, pi, ELDER_K_RESIDUAL, G, 8, 8, S, st, -1, mixed);
     launch_norm_finalize(ctx->partial, ctx->partial2, nb, ns, 0, S, st);
     CKL();
 
@@ -1443,7 +1449,7 @@ int step_impl(elder_ctx* ctx, int S, const double* phi, const double* K, double*
             launch_residual(G, ph, ctx->bc[0], ctx->cval, phi, K, ctx->pt, ctx->ct, ctx->p_old,
                             ctx->c_old, ctx->Rt, ctx->partial, ctx->partial3, lsmask, NSTRIDE,
                             S, st, ctx->qf, mixed);
-            prof_end(ctx, pi, ELDER_K_RESIDUAL, G, 8, 8, ctx->n_active_ls, st);
+            prof_end(ctx, pi, ELDER_K_RESIDUAL, G, 8, 8, ctx->n_active_ls, st, -1, mixed);
             launch_norm_finalize(ctx->partial, ctx->partial3, nb, ns, 1, S, st);
             launch_newton_ls_finalize(nullptr, ctx->partial2, nb, ns, set.ls_max, S, st);
             CKL();
