@@ -469,7 +469,6 @@ def run_ours(a):
     pk = prof[top]
     peaks = measured_peaks()
     hbm_peak = peaks["hbm_gbs"] if peaks else 6800.0
-    tsize = 4 if a.precision == "mixed" else 8
     per_launch_ms = pk["ms"] / max(pk["launches"], 1)
     bytes_per_launch = pk["bytes"] / max(pk["launches"], 1)
     # the mixed solver's finest level under the z-line smoother stores no matrix
@@ -498,10 +497,7 @@ def run_ours(a):
                 "frac": achieved / peak if achieved else None,
                 "peak_source": src,
                 "traffic": (tr * bytes_per_launch /
-                            max(1e-30, E_model_bytes(top, tsize, nx, ny, nz,
-                                                     a.smoother != "jacobi",
-                                                     ilu=a.smoother == "ilu",
-                                                     matrix_free=mf_top))
+                            max(1e-30, launch_model_bytes(a, top))
                             if tr is not None else None),
                 "algorithmic_flops_per_launch": pk["flops"] / max(pk["launches"], 1),
                 "algorithmic_bytes_per_launch": bytes_per_launch, "avg_launch_ms": per_launch_ms,
@@ -793,32 +789,52 @@ def gpc_timings(E, torch, cfield, stream, Ns=1_000_000, apk=None):
     return res
 
 
-def E_model_bytes(cls, tsize, nx, ny, nz, line=True, ilu=False, matrix_free=False):
+def launch_model_bytes(a, cls):
+    """Algorithmic bytes per node of one launch of a class on the finest level of
+    the solver that the arguments ask for: elder_profile_read's model."""
+    mixed = a.precision == "mixed"
+    # (the assembly forms the line factors under every smoother, up to nz = 128)
+    line = a.grid[2] <= 128 if cls == "jacobian" else a.smoother != "jacobi"
+    return E_model_bytes(cls, 4 if mixed else 8, *a.grid, line=line, ilu=a.smoother == "ilu",
+                         matrix_free=mixed and a.smoother == "zline", line_factors=3)
+
+
+def E_model_bytes(cls, tsize, nx, ny, nz, line=True, ilu=False, matrix_free=False,
+                  line_factors=2):
     """Algorithmic bytes per node of one launch on a level with a stored matrix
-    (bfloat16 multigrid matrices in the mixed path); matrix_free: the Krylov
-    products and the multigrid residual of the mixed solver's finest level, from
-    the state, the coefficients and the vectors.  With the z-line
-    smoother the sweep from x = 0 reads line factors (zMi, zC),
-    the lower line block, b and writes x; the assembly also forms those
-    factors (reading Dinv and both line blocks).  With the ILU smoother
-    (ilu=True) the sweep from x = 0 reads the 26 factor blocks, the inverse
-    pivot, b and bc twice, writes, reads and rewrites its scratch vector and
-    writes x; the assembly also forms the factors (J, Dinv, bc read; 26
+    (bfloat16 multigrid matrices in the mixed path); matrix_free: on the mixed
+    solver's finest level under the z-line smoother, from the state, the
+    coefficients and the vectors, line blocks in FP32.  The z-line sweep from
+    x = 0 reads b and line_factors blocks per node and writes x: 3, the library's
+    zMi, zA and zC; 2, zMi and zC beside the matrix's own lower block.  The
+    assembly also forms those factors (reading Dinv and both line blocks).  With
+    the ILU smoother (ilu=True) the sweep from x = 0 reads the 26 factor blocks,
+    the inverse pivot, b and bc twice, writes, reads and rewrites its scratch
+    vector and writes x; the assembly also forms the factors (J, Dinv, bc read; 26
     factor blocks and the inverse pivot written)."""
     N = (nx + 1) * (ny + 1) * (nz + 1)
     cpn = nx * ny * nz / N
     mz = 2 if tsize == 4 else 8
-    if matrix_free and cls in ("spmv", "mg_residual"):
-        return 8 * tsize + 2 * tsize * cpn + 1
-    smooth0 = (12 * tsize + 4 * mz + 1) if line else 8 * tsize + 1
+    factors = 4 * line_factors * tsize
+    smooth0 = factors + 4 * tsize + (4 * mz if line_factors == 2 else 0) + 1
+    if not line:
+        smooth0 = 8 * tsize + 1
     if ilu:
         smooth0 = 104 * mz + 14 * tsize + 2
+    if matrix_free and cls in ("spmv", "mg_residual"):
+        return 8 * tsize + 2 * tsize * cpn + 1
+    if matrix_free and cls == "smooth":
+        return 26 * tsize + 2 * tsize * cpn + 2
+    if matrix_free and cls == "jacobian":
+        return 40 * tsize + 18 + 2 * tsize * cpn
     return {"smooth": 108 * mz + 10 * tsize + 1,
             "smooth0": smooth0,
             "spmv": 108 * tsize + 6 * tsize + 1, "mg_residual": 108 * mz + 6 * tsize + 1,
             "residual": 49 + 16 * cpn,
-            "jacobian": 108 * tsize + 108 * mz + 4 * tsize + 17 + 16 * cpn +
-                        ((12 * tsize + 8 * mz + 1) if line else 0) +
+            # (the Krylov copy and the multigrid copy: one array in FP64)
+            "jacobian": (108 * tsize if tsize == 4 else 0) + 108 * mz + 4 * tsize + 17 +
+                        16 * cpn +
+                        ((factors + 4 * tsize + 8 * mz + 1) if line else 0) +
                         ((212 * mz + 8 * tsize + 1) if ilu else 0)}[cls]
 
 

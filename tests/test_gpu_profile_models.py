@@ -58,3 +58,35 @@ def test_fp64(E):
     r, j = prof[E.K_RESIDUAL], prof[E.K_JACOBIAN]
     _is_multiple(r["flops"], 266 * C + 75 * nodes[0], r["launches"])
     _is_multiple(j["flops"], 2890 * sum(nodes), j["launches"] / len(nodes))
+
+
+@pytest.mark.parametrize("precision", ["mixed", "fp64"])
+@pytest.mark.parametrize("smoother", ["zline", "jacobi", "ilu"])
+@pytest.mark.parametrize("levels", [0, 1])
+def test_bench_model_is_the_library_s(E, precision, smoother, levels):
+    """bench.launch_model_bytes of the finest level against the bytes counted: the
+    Krylov products run there only; on a single-level grid so does the assembly
+    (with rows: a matrix-free level lies above a coarser one)."""
+    import argparse
+
+    import bench
+    dims = (6, 4, 2)
+    a = argparse.Namespace(precision=precision, smoother=smoother, grid=list(dims))
+    ctx = E.elder_create(E.elder_config_default(
+        *dims, precision=E.ELDER_MIXED if precision == "mixed" else E.ELDER_FP64, bc_mode=2,
+        mg_levels=levels,
+        smoother={"zline": E.ELDER_SMOOTH_ZLINE, "jacobi": E.ELDER_SMOOTH_JACOBI,
+                  "ilu": E.ELDER_SMOOTH_ILU}[smoother]))
+    assert ctx.levels == (1 if levels else 2)
+    p, c = ctx.initial_state(1)
+    phi = torch.full((ctx.C,), 0.1, dtype=torch.float64, device="cuda:0")
+    ctx.profile(True)
+    ctx.step(1, phi, torch.full_like(phi, 4.845e-13), p, c, E.SECONDS_PER_YEAR / 48)
+    ctx.profile(False)
+    spmv, jac = ctx.profile_read(E.K_SPMV), ctx.profile_read(E.K_JACOBIAN)
+    ctx.destroy()
+    if levels == 0:
+        _is_multiple(spmv["bytes"], bench.launch_model_bytes(a, "spmv") * 105, spmv["launches"])
+    elif smoother != "ilu":  # (no ILU factors on the coarsest level)
+        a.smoother = "jacobi"  # the rows' model
+        _is_multiple(jac["bytes"], bench.launch_model_bytes(a, "jacobian") * 105, jac["launches"])
