@@ -1006,11 +1006,13 @@ __device__ __forceinline__ unsigned gj_key(float a)
 {
     return min(__float_as_uint(a) & 0x7fffffffu, 0x7f800000u);
 }
-// the warp's maximum, for each lane whether its key is equal to it
+// The warp's maximum, for each lane whether its key is equal to it.  Each reduction
+// waits for all lanes of its mask: every lane takes part in both, whatever the first
+// one gave it (behind `top &&` the lanes without the largest high word would skip the
+// second, and the warp would never get past it).
 __device__ __forceinline__ bool gj_is_max(unsigned long long key)
 {
     const unsigned hi = (unsigned)(key >> 32), lo = (unsigned)key;
-    // (every lane takes part in both reductions)
     const bool top = hi == __reduce_max_sync(0xffffffffu, hi);
     const unsigned low = __reduce_max_sync(0xffffffffu, top ? lo : 0u);
     return top && lo == low;

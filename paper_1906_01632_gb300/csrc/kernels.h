@@ -70,13 +70,14 @@ constexpr int kMaxBS = 512;  // largest block of the autotuned stencil kernels
 constexpr int kMinBS = 128;  // smallest block of the autotuned stencil kernels
 
 inline int nblocks(int n, int bs = kBS) { return (n + bs - 1) / bs; }
+constexpr int kSMs = 152;    // of the GB300, the one target
 // Threads per block of a launch over n items of S samples: bs, halved down to
 // a warp while the launch has fewer blocks than two per SM.  On small grids a
 // block of 256 threads serialises its FP64 work on one SM while others idle:
 // the FP64 multigrid residual of a 32x32x8 sample (39 blocks) took 20 us.
 inline int spread_block(int bs, int n, int S)
 {
-    while (bs > 32 && (long long)nblocks(n, bs) * S < 304) bs /= 2;
+    while (bs > 32 && (long long)nblocks(n, bs) * S < 2 * kSMs) bs /= 2;
     return bs;
 }
 // blocks of the BiCGStab x/r update (4 nodes per thread): its partials per sample

@@ -118,8 +118,7 @@ __device__ __forceinline__ void plane31(float2 (&q)[4])
 }
 
 // The four corners (x + 2 z) of one row of a cell column, p = (p', x_p) and c =
-// (c, x_c), and the row's in-plane sums: gx[z], gz[x] the (3,1) sums of the x
-// and z differences of p, C the (3,1) x (3,1) sums of c.
+// (c, x_c).
 struct MfRow {
     float2 p[4], c[4];
 };
@@ -413,8 +412,12 @@ MfTiling choose_tiling(const Grid& G, int S)
         }
     }
     // chunks of rows: each adds a layer (and a start of about one more); the
-    // launch's time goes with its waves times the layers of a chunk
-    const int slots = 152 * std::max(1, kMfResident / best.threads);
+    // launch's time goes with its waves times the layers of a chunk.  They follow
+    // from the batch, and with them which rows a partial of the inner products
+    // adds up: the values of y do not depend on them, the last bits of the FP64
+    // sums do (partials of fixed groups of rows made the mixed steps 1 to 8 %
+    // slower)
+    const int slots = kSMs * std::max(1, kMfResident / best.threads);
     double lt = 1e300;
     const int base = best.ntx * best.ntz * S;
     for (int nch = 1; nch <= std::max(1, ny1 / 3); ++nch) {
